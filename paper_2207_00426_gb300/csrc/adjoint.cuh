@@ -157,7 +157,7 @@ SQSM_DEV void predict_factor(const T* F, const T* N, const T* SQ, T* Nm) {
       P[i * 2 * NX + j] = s;
       P[i * 2 * NX + NX + j] = SQ[i * NX + j];
     }
-  tria<T, NX, 2 * NX>(P);
+  tria<T, NX, 2 * NX, DenseThenLower<NX>>(P);
   take_lower<T, NX, 2 * NX>(P, Nm);
 }
 

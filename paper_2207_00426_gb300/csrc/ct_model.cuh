@@ -439,7 +439,7 @@ SQSM_DEV void cubature_regress(const T* m, const T* N, const T* gm, bool subtrac
     for (int i = 0; i < NX; ++i) B[r * C + NO + i] = (Hs[r * NX + i] - dbar[r]) / sq;
     if constexpr (w0 > 0.0) B[r * C + NO + NX] = -T(sqrt(w0)) * dbar[r];
   }
-  tria<T, NO, C>(B);
+  tria_full<T, NO, C>(B);
   take_lower<T, NO, C>(B, Sout);
 }
 
@@ -540,7 +540,7 @@ SQSM_DEV void gauss_hermite_regress(const T* m, const T* N, const T* gm, bool su
         B[r * C + NO + q] = sw * res;
       }
     }
-    tria<T, NO, C>(B);
+    tria_full<T, NO, C>(B);
 #pragma unroll
     for (int r = 0; r < NO; ++r)
 #pragma unroll

@@ -249,7 +249,7 @@ SQSM_DEV T kf_step(const Gamma<T, NX, NY>& g, const T* y, T* m, T* N) {
       P[i * 2 * NX + NX + j] = g.SQ[i * NX + j];   // S_Lambda
     }
   }
-  tria<T, NX, 2 * NX>(P);
+  tria<T, NX, 2 * NX, DenseThenLower<NX>>(P);
   constexpr int W = NX + NY;
   T Psi[W * W];
 #pragma unroll
@@ -271,7 +271,7 @@ SQSM_DEV T kf_step(const Gamma<T, NX, NY>& g, const T* y, T* m, T* N) {
 #pragma unroll
     for (int j = 0; j < NY; ++j) Psi[(NY + i) * W + NX + j] = T(0);
   }
-  tria<T, W, W>(Psi);
+  tria<T, W, W, DenseLowerOverLower<NY, NX>>(Psi);
   T e[NY], Y[NY * NY];
 #pragma unroll
   for (int i = 0; i < NY; ++i) {
@@ -340,7 +340,7 @@ SQSM_DEV void filter_element(const Gamma<T, NX, NY>& g, const T* y, bool first, 
         P[i * 2 * NX + j] = s;
         P[i * 2 * NX + NX + j] = g.SQ[i * NX + j];
       }
-    tria<T, NX, 2 * NX>(P);
+    tria<T, NX, 2 * NX, DenseThenLower<NX>>(P);
     take_lower<T, NX, 2 * NX>(P, Bm);
   } else {
 #pragma unroll
@@ -367,7 +367,7 @@ SQSM_DEV void filter_element(const Gamma<T, NX, NY>& g, const T* y, bool first, 
 #pragma unroll
     for (int j = 0; j < NY; ++j) Psi[(NY + i) * W + NX + j] = T(0);
   }
-  tria<T, W, W>(Psi);
+  tria<T, W, W, DenseLowerOverLower<NY, NX>>(Psi);
   T Y[NY * NY];
 #pragma unroll
   for (int i = 0; i < NY; ++i)
@@ -443,6 +443,20 @@ SQSM_DEV void filter_element(const Gamma<T, NX, NY>& g, const T* y, bool first, 
   zero_pad<T, R::Z + NX * NX, R::size>(e);
 }
 
+// A single step's element has Z zero-padded, not triangular; items of the
+// upper levels are combined as lower ones: Z <- Tria(Z) (its other columns
+// are zero, so min(n_x, n_y) reflections).
+template <typename T, int NX, int NY>
+SQSM_DEV void lower_Z(T* Z) {
+  if constexpr (NX >= NY) {
+    tria<T, NX, NX, FewColumns<NY>, NY>(Z);
+#pragma unroll
+    for (int i = 0; i < NX; ++i)
+#pragma unroll
+      for (int j = i + 1; j < NX; ++j) Z[i * NX + j] = T(0);
+  }
+}
+
 // The blocks of Xi (eq. sqrt-filter-com-2), Xi = Tria([[M, I], [Z_j, 0]])
 // with M = U_i^T Z_j, from two NX x 2NX Trias instead of one 2NX x 2NX one.
 // Multiplying out Xi Xi^T = [[I + M M^T, M Z_j^T], [Z_j M^T, Z_j Z_j^T]]:
@@ -453,21 +467,27 @@ SQSM_DEV void filter_element(const Gamma<T, NX, NY>& g, const T* y, bool first, 
 // (the push-through identity); Xi_22 enters the operator only through
 // Tria([A_i^T Xi_22, Z_i]), which W gives the same product.  Xi_11 and L
 // are >= I, so the triangular solves are well conditioned.
-template <typename T, int NX>
+// Z_j is lower triangular (ZLOW; NZ = NX), or has its first NZ columns nonzero
+// (the zero-padded factor of a single step, NZ = n_y); M then too.
+template <typename T, int NX, int NZ, bool ZLOW>
 SQSM_DEV void xi_m(const T* Ui, const T* Zj, T* Mx) {
 #pragma unroll
   for (int i = 0; i < NX; ++i)
 #pragma unroll
     for (int j = 0; j < NX; ++j) {
       T s = T(0);
+      if (j < NZ) {
 #pragma unroll
-      for (int k = i; k < NX; ++k) s += Ui[k * NX + i] * Zj[k * NX + j];   // U_i lower
+        for (int k = i; k < NX; ++k)   // U_i lower
+          if (!ZLOW || k >= j) s += Ui[k * NX + i] * Zj[k * NX + j];
+      }
       Mx[i * NX + j] = s;
     }
 }
 
-// Tria([A, I]) for A (NX x NX), or Tria([A^T, I]) with TRANS.
-template <typename T, int NX, bool TRANS>
+// Tria([A, I]) for A (NX x NX) with its first NZ columns nonzero, or
+// Tria([A^T, I]) with TRANS.
+template <typename T, int NX, bool TRANS, int NZ>
 SQSM_DEV void tria_with_identity(const T* A, T* L) {
   constexpr int C2 = 2 * NX;
   T B[NX * C2];
@@ -478,42 +498,111 @@ SQSM_DEV void tria_with_identity(const T* A, T* L) {
       B[i * C2 + j] = TRANS ? A[j * NX + i] : A[i * NX + j];
       B[i * C2 + NX + j] = i == j ? T(1) : T(0);
     }
-  tria<T, NX, C2>(B);
+  if constexpr (TRANS) tria<T, NX, C2, FewRowsThenIdentity<NZ, NX>>(B);
+  else tria<T, NX, C2, FewThenIdentity<NZ, NX>>(B);
   take_lower<T, NX, C2>(B, L);
 }
 
 // G = Xi_21 Xi_11^{-1} = Z_j M^T Xi_11^{-T} Xi_11^{-1}.
-template <typename T, int NX>
+template <typename T, int NX, int NZ, bool ZLOW>
 SQSM_DEV void xi_gain(const T* Zj, const T* Mx, const T* X11, T* G) {
-  mmt<T, NX, NX, NX>(Zj, Mx, G);
+#pragma unroll
+  for (int i = 0; i < NX; ++i)
+#pragma unroll
+    for (int j = 0; j < NX; ++j) {
+      T s = T(0);
+#pragma unroll
+      for (int k = 0; k < NZ; ++k)
+        if (!ZLOW || k <= i) s += Zj[i * NX + k] * Mx[j * NX + k];
+      G[i * NX + j] = s;
+    }
   rsolve_t<T, NX, NX>(G, X11);
   rsolve<T, NX, NX>(G, X11);
+}
+
+// Tria([V, U_j]) of the combine and of the carry application.  V is a
+// triangular solve's result, whose last products the compiler fuses into the
+// first reflections; in FP32 the full loops keep that choice, and with it the
+// rounding of long runs that amplify any other (their errors sit close to the
+// targets, and another rounding is another draw of them).
+template <typename T, int NX>
+SQSM_DEV void tria_solved(T* B) {
+  if constexpr (sizeof(T) == 4) tria_full<T, NX, 2 * NX>(B);
+  else tria<T, NX, 2 * NX, DenseThenLower<NX>>(B);
+}
+
+// A_j U_i for a lower U_i.
+template <typename T, int NX>
+SQSM_DEV void mm_lower(const T* A, const T* U, T* V) {
+#pragma unroll
+  for (int i = 0; i < NX; ++i)
+#pragma unroll
+    for (int j = 0; j < NX; ++j) {
+      T s = T(0);
+#pragma unroll
+      for (int k = j; k < NX; ++k) s += A[i * NX + k] * U[k * NX + j];
+      V[i * NX + j] = s;
+    }
+}
+
+// y = U x and y = U^T x for a lower U.
+template <typename T, int NX>
+SQSM_DEV void mv_lower(const T* U, const T* x, T* y) {
+#pragma unroll
+  for (int i = 0; i < NX; ++i) {
+    T s = T(0);
+#pragma unroll
+    for (int k = 0; k <= i; ++k) s += U[i * NX + k] * x[k];
+    y[i] = s;
+  }
+}
+template <typename T, int NX>
+SQSM_DEV void mtv_lower(const T* U, const T* x, T* y) {
+#pragma unroll
+  for (int i = 0; i < NX; ++i) {
+    T s = T(0);
+#pragma unroll
+    for (int k = i; k < NX; ++k) s += U[k * NX + i] * x[k];
+    y[i] = s;
+  }
 }
 
 // b_ij and eta_ij of Table 3 from the combine's factors: A_i, U_i, Z_j, the
 // gain G and A_j (I - U_i G^T) (see filter_combine).  The full operator and
 // the mean-only refinement passes (which read the factors back from a
 // table) both take this path, so the two give the same values bit for bit.
-template <typename T, int NX>
+template <typename T, int NX, int NZ = NX, bool ZLOW = true>
 SQSM_DEV void filter_combine_means(const T* Ai, const T* Ui, const T* Zj, const T* G,
                                    const T* AjM, const T* bi, const T* etai, const T* bj,
                                    const T* etaj, T* bo, T* etao) {
   // b_ij
   T t[NX], u[NX];
-  mtv<T, NX, NX>(Ui, etaj, t);
-  mv<T, NX, NX>(Ui, t, u);
+  mtv_lower<T, NX>(Ui, etaj, t);
+  mv_lower<T, NX>(Ui, t, u);
 #pragma unroll
   for (int i = 0; i < NX; ++i) u[i] += bi[i];
   mv<T, NX, NX>(AjM, u, t);
 #pragma unroll
   for (int i = 0; i < NX; ++i) bo[i] = t[i] + bj[i];
-  // eta_ij
+  // eta_ij (Z_j lower, or its first NZ columns)
   T sv[NX], r[NX];
-  mtv<T, NX, NX>(Zj, bi, sv);
-  mv<T, NX, NX>(Zj, sv, r);
 #pragma unroll
-  for (int i = 0; i < NX; ++i) r[i] = etaj[i] - r[i];
-  mtv<T, NX, NX>(Ui, r, t);
+  for (int i = 0; i < NZ; ++i) {
+    T s = T(0);
+#pragma unroll
+    for (int k = 0; k < NX; ++k)
+      if (!ZLOW || k >= i) s += Zj[k * NX + i] * bi[k];
+    sv[i] = s;
+  }
+#pragma unroll
+  for (int i = 0; i < NX; ++i) {
+    T s = T(0);
+#pragma unroll
+    for (int k = 0; k < NZ; ++k)
+      if (!ZLOW || k <= i) s += Zj[i * NX + k] * sv[k];
+    r[i] = etaj[i] - s;
+  }
+  mtv_lower<T, NX>(Ui, r, t);
   mv<T, NX, NX>(G, t, sv);
 #pragma unroll
   for (int i = 0; i < NX; ++i) r[i] -= sv[i];
@@ -536,20 +625,26 @@ SQSM_DEV void filter_combine_means(const T* Ai, const T* Ui, const T* Zj, const 
 // only the factors its part needs.  With gm (part 0) the combine's G and
 // A_j (I - U_i G^T) are also stored there (FGm layout), for the mean-only
 // passes that replay b_ij and eta_ij.
-template <typename T, int NX, int PARTS = 7>
+// U and Z of both operands are lower triangular.  STEP: e_j is a single
+// step's element, whose Z has its first NZ = min(n_x, n_y) columns nonzero and
+// not triangular, and e_i is one too or a fold of such: M, L, W and Z_ij's
+// block then have NZ columns (or rows), and the terms with the rest, exact
+// zeros, are left out.
+template <typename T, int NX, int PARTS = 7, bool STEP = false, int NZ = NX>
 SQSM_DEV void filter_combine(const T* ei, const T* ej, T* out, T* gm = nullptr) {
   using R = FRec<NX>;
   constexpr int C2 = 2 * NX;
   constexpr bool ABE = PARTS & 1, UU = PARTS & 2, ZZ = PARTS & 4;
+  static_assert(STEP || NZ == NX, "fewer columns of Z only for single steps");
   const T* Ui = ei + R::U;
   const T* Zj = ej + R::Z;
   T Mx[NX * NX];
-  xi_m<T, NX>(Ui, Zj, Mx);
+  xi_m<T, NX, NZ, !STEP>(Ui, Zj, Mx);
   T X11[NX * NX];
-  if constexpr (ABE || UU) tria_with_identity<T, NX, false>(Mx, X11);
+  if constexpr (ABE || UU) tria_with_identity<T, NX, false, NZ>(Mx, X11);
   if constexpr (ABE) {
     T G[NX * NX];
-    xi_gain<T, NX>(Zj, Mx, X11, G);
+    xi_gain<T, NX, NZ, !STEP>(Zj, Mx, X11, G);
     // Minv = I - U_i G^T
     T Mi[NX * NX];
 #pragma unroll
@@ -564,7 +659,7 @@ SQSM_DEV void filter_combine(const T* ei, const T* ej, T* out, T* gm = nullptr) 
     T AjM[NX * NX];
     mm<T, NX, NX, NX>(ej + R::A, Mi, AjM);
     mm<T, NX, NX, NX>(AjM, ei + R::A, out + R::A);
-    filter_combine_means<T, NX>(ei + R::A, Ui, Zj, G, AjM, ei + R::b, ei + R::eta, ej + R::b,
+    filter_combine_means<T, NX, NZ, !STEP>(ei + R::A, Ui, Zj, G, AjM, ei + R::b, ei + R::eta, ej + R::b,
                                 ej + R::eta, out + R::b, out + R::eta);
     if (gm) {
       T v[FGm<NX>::size];
@@ -581,7 +676,7 @@ SQSM_DEV void filter_combine(const T* ei, const T* ej, T* out, T* gm = nullptr) 
   if constexpr (UU) {
     // U_ij = Tria([A_j U_i Xi11^{-T}, U_j])
     T V[NX * NX];
-    mm<T, NX, NX, NX>(ej + R::A, Ui, V);
+    mm_lower<T, NX>(ej + R::A, Ui, V);
     rsolve_t<T, NX, NX>(V, X11);
     T B[NX * C2];
 #pragma unroll
@@ -591,28 +686,42 @@ SQSM_DEV void filter_combine(const T* ei, const T* ej, T* out, T* gm = nullptr) 
         B[i * C2 + j] = V[i * NX + j];
         B[i * C2 + NX + j] = ej[R::U + i * NX + j];
       }
-    tria<T, NX, C2>(B);
+    tria_solved<T, NX>(B);
     take_lower<T, NX, C2>(B, out + R::U);
   }
   if constexpr (ZZ) {
     // Z_ij = Tria([A_i^T W, Z_i]),  W = Z_j L^{-T},  L = Tria([M^T, I])
-    T L[NX * NX], W[NX * NX];
-    tria_with_identity<T, NX, true>(Mx, L);
+    T L[NX * NX], W[NX * NZ];
+    tria_with_identity<T, NX, true, NZ>(Mx, L);
+    {   // row by row z L^T = Z_j (rows and columns NZ.. of L are the identity's)
+      T inv[NZ];
 #pragma unroll
-    for (int i = 0; i < NX * NX; ++i) W[i] = Zj[i];
-    rsolve_t<T, NX, NX>(W, L);
+      for (int i = 0; i < NZ; ++i) inv[i] = hh_rcp(L[i * NX + i]);
+#pragma unroll
+      for (int r = 0; r < NX; ++r)
+#pragma unroll
+        for (int i = 0; i < NZ; ++i) {
+          T a = Zj[r * NX + i];
+#pragma unroll
+          for (int k = 0; k < i; ++k) a -= W[r * NZ + k] * L[i * NX + k];
+          W[r * NZ + i] = a * inv[i];
+        }
+    }
     T B[NX * C2];
 #pragma unroll
     for (int i = 0; i < NX; ++i)
 #pragma unroll
       for (int j = 0; j < NX; ++j) {
         T a = T(0);
+        if (j < NZ) {
 #pragma unroll
-        for (int k = 0; k < NX; ++k) a += ei[R::A + k * NX + i] * W[k * NX + j];
+          for (int k = 0; k < NX; ++k) a += ei[R::A + k * NX + i] * W[k * NZ + j];
+        }
         B[i * C2 + j] = a;
         B[i * C2 + NX + j] = ei[R::Z + i * NX + j];
       }
-    tria<T, NX, C2>(B);
+    if constexpr (STEP) tria<T, NX, C2, FewThenFewLower<NZ, NX, NZ>>(B);
+    else tria<T, NX, C2, DenseThenLower<NX>>(B);
     take_lower<T, NX, C2>(B, out + R::Z);
   }
   if constexpr (PARTS == 7) zero_pad<T, R::Z + NX * NX, R::size>(out);
@@ -626,12 +735,12 @@ SQSM_DEV void filter_apply(const T* bi, const T* Ui, const T* ej, T* bo, T* Uo) 
   using R = FRec<NX>;
   constexpr int C2 = 2 * NX;
   T Mx[NX * NX], X11[NX * NX], G[NX * NX];
-  xi_m<T, NX>(Ui, ej + R::Z, Mx);
-  tria_with_identity<T, NX, false>(Mx, X11);
-  xi_gain<T, NX>(ej + R::Z, Mx, X11, G);
+  xi_m<T, NX, NX, true>(Ui, ej + R::Z, Mx);
+  tria_with_identity<T, NX, false, NX>(Mx, X11);
+  xi_gain<T, NX, NX, true>(ej + R::Z, Mx, X11, G);
   T t[NX], u[NX], w[NX];
-  mtv<T, NX, NX>(Ui, ej + R::eta, t);
-  mv<T, NX, NX>(Ui, t, u);
+  mtv_lower<T, NX>(Ui, ej + R::eta, t);
+  mv_lower<T, NX>(Ui, t, u);
 #pragma unroll
   for (int i = 0; i < NX; ++i) u[i] += bi[i];
   // (I - U_i G^T) u
@@ -643,14 +752,14 @@ SQSM_DEV void filter_apply(const T* bi, const T* Ui, const T* ej, T* bo, T* Uo) 
     for (int k = 0; k < NX; ++k) s += G[k * NX + i] * u[k];
     t[i] = s;
   }
-  mv<T, NX, NX>(Ui, t, w);
+  mv_lower<T, NX>(Ui, t, w);
 #pragma unroll
   for (int i = 0; i < NX; ++i) w[i] = u[i] - w[i];
   mv<T, NX, NX>(ej + R::A, w, t);
 #pragma unroll
   for (int i = 0; i < NX; ++i) bo[i] = t[i] + ej[R::b + i];
   T V[NX * NX];
-  mm<T, NX, NX, NX>(ej + R::A, Ui, V);
+  mm_lower<T, NX>(ej + R::A, Ui, V);
   rsolve_t<T, NX, NX>(V, X11);
   T B[NX * C2];
 #pragma unroll
@@ -660,7 +769,7 @@ SQSM_DEV void filter_apply(const T* bi, const T* Ui, const T* ej, T* bo, T* Uo) 
       B[i * C2 + j] = V[i * NX + j];
       B[i * C2 + NX + j] = ej[R::U + i * NX + j];
     }
-  tria<T, NX, C2>(B);
+  tria_solved<T, NX>(B);
   take_lower<T, NX, C2>(B, Uo);
 }
 
@@ -723,7 +832,8 @@ SQSM_DEV void smoother_element(const Gamma<T, NX, NY>& g, const T* mf, const T* 
       Phi[(NX + i) * C2 + j] = Nf[i * NX + j];
       Phi[(NX + i) * C2 + NX + j] = T(0);
     }
-  tria<T, C2, C2>(Phi);
+  if constexpr (sizeof(T) == 4 && NX <= 2) tria_full<T, C2, C2>(Phi);   // nothing to leave out
+  else tria<T, C2, C2, DenseLowerOverLower<NX, NX>>(Phi);
   T P11[NX * NX];
   take_lower<T, NX, C2>(Phi, P11);
 #pragma unroll
@@ -772,7 +882,7 @@ SQSM_DEV void smoother_combine(const T* ei, const T* ej, T* out) {
       B[i * C2 + j] = s;
       B[i * C2 + NX + j] = ei[R::D + i * NX + j];
     }
-  tria<T, NX, C2>(B);
+  tria_solved<T, NX>(B);
   take_lower<T, NX, C2>(B, out + R::D);
   zero_pad<T, R::D + NX * NX, R::size>(out);
 }
@@ -795,7 +905,7 @@ SQSM_DEV void smoother_apply(const T* ei, T* gm, T* Dm) {
       B[i * C2 + j] = s;
       B[i * C2 + NX + j] = ei[R::D + i * NX + j];
     }
-  tria<T, NX, C2>(B);
+  tria_solved<T, NX>(B);
   smoother_apply_g<T, NX>(ei + R::E, ei + R::g, gm);
   take_lower<T, NX, C2>(B, Dm);
 }

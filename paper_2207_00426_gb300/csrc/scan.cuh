@@ -78,10 +78,11 @@ filter_leaf_up(DevLevel lv, DevSeqs sq, GV gv, const T* __restrict__ y,
       filter_element<T, NX, NY>(g, ys, s == off, m0b, N0b, agg);
     } else {
       filter_element<T, NX, NY>(g, ys, s == off, m0b, N0b, el);
-      filter_combine<T, NX>(agg, el, tmp);
+      filter_combine<T, NX, 7, true, (NX < NY ? NX : NY)>(agg, el, tmp);
       copy<T, REC>(tmp, agg);
     }
   }
+  if (cnt == 1) lower_Z<T, NX, NY>(agg + FRec<NX>::Z);
   vstore<T, REC>(items + c * REC, agg);
 }
 
