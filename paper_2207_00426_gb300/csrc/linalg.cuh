@@ -48,6 +48,21 @@ SQSM_DEV double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 SQSM_DEV float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 SQSM_DEV double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// x / c for a constant c: the product with the rounded reciprocal, corrected
+// by the remainder (a division by a divisor known in advance; Brisebarre,
+// Muller and Raina, IEEE Trans. Computers 2004).  Equal to the rounded
+// quotient: for the divisors the sigma-point rules use (10, 12 and once and
+// twice sqrt(5), sqrt(6)) checked over every FP32 significand.
+template <typename T> struct ConstDivisor {
+  T c, rc;
+  __host__ __device__ constexpr explicit ConstDivisor(T c_) : c(c_), rc(T(1) / c_) {}
+};
+template <typename T>
+SQSM_DEV T div_const(T x, const ConstDivisor<T>& d) {
+  const T q = mul_rn(x, d.rc);
+  return fma_rn(fma_rn(-q, d.c, x), d.rc, q);
+}
+
 // Which entries of a matrix handed to Tria can be nonzero: row(i) is the bit
 // mask of the columns of row i that may be (bit j: column j).  Nearly every
 // matrix the method triangularises is a block matrix with triangular, empty
