@@ -64,6 +64,7 @@ struct Plan {
   Alloc mem;
   int B = 0;
   int L0 = 0, R = 0;
+  bool lanes = false;   // adaptive levels in the lane forms (FP64)
   std::vector<int64_t> offsets;
   int64_t* d_offsets = nullptr;
   LevelSet filt, smth;
@@ -153,13 +154,25 @@ int cuda_fail(sqsm_ctx* ctx, cudaError_t e, const char* where) {
 // to fill the GPU.
 constexpr int64_t kFoldAboveItems = 160000;
 
+// FP64 plans (lane forms): a level with more items than this is folded 4 per
+// thread, whose instructions then fill enough warps to keep every FP64 unit
+// busy (160 warps, one per SM); one with fewer is folded 4 per lane group,
+// whose combine issues a fifth of the instructions per warp but uses a
+// sixteenth of the warp; one that fits one block of Kogge-Stone chunks per
+// SM is scanned in such chunks.  Two iterations with one step per leaf,
+// n = 16000: 1.94 ms against 2.36 folded per thread; at n = 1e5 the two forms
+// are even.
+constexpr int64_t kLaneMaxItems = 20000;
+
 // Levels of a segmented scan whose level-0 items are `counts[b]` per
 // sequence: chunks of L0 items at the leaf, then chunks of R items (or, for
 // R == 0, of 4 or 32 items chosen per level) until each sequence has one item.
 
-bool build_levels(Plan& p, const std::vector<int64_t>& counts0, LevelSet& L) {
+bool build_levels(Plan& p, const std::vector<int64_t>& counts0, LevelSet& L, int sm_count,
+                  int lane_chunk) {
   std::vector<int64_t> counts = counts0;
   L.B = (int)counts0.size();
+  L.lanes = p.lanes;
   int level = 0;
   int64_t total = 0;
   for (int64_t v : counts) total += v;
@@ -168,14 +181,21 @@ bool build_levels(Plan& p, const std::vector<int64_t>& counts0, LevelSet& L) {
   for (;;) {
     int64_t size = level == 0 ? p.L0 : p.R;
     if (level > 0) {
-      bool cs = false;
+      char form = kFoldLevel;
       if (p.R == 0) {                       // adaptive: see get_plan
         int64_t items = 0;
         for (int64_t v : counts) items += v;
-        cs = items <= kFoldAboveItems;
-        size = cs ? kChunkScan : 4;
+        if (p.lanes)
+          form = items > kLaneMaxItems                      ? kFoldLevel
+                 : items > int64_t(sm_count) * lane_chunk   ? kLaneFoldLevel
+                                                            : kLaneChunkLevel;
+        else
+          form = items <= kFoldAboveItems ? kChunkLevel : kFoldLevel;
+        size = form == kChunkLevel ? kChunkScan
+               : form == kLaneChunkLevel ? lane_chunk
+               : form == kLaneFoldLevel ? kLaneFold : 4;
       }
-      L.cs.push_back(cs ? 1 : 0);
+      L.cs.push_back(form);
     }
     std::vector<int64_t> first;
     std::vector<int32_t> count, seq;
@@ -240,6 +260,11 @@ bool build_levels(Plan& p, const std::vector<int64_t>& counts0, LevelSet& L) {
   return true;
 }
 
+// Calls whose adaptive upper levels take the lane forms.
+bool lane_plan(int dtype, int nx, int R) {
+  return dtype == SQSM_F64 && nx >= kLaneMinNx && R == 0;
+}
+
 // Scan shape from the options, else the default: leaf 3 steps per thread
 // while the leaf chunks fit one wave of the leaf kernels (256 threads per SM
 // at their register use), so that the latency-bound leaf chains are short, 4
@@ -248,16 +273,22 @@ bool build_levels(Plan& p, const std::vector<int64_t>& counts0, LevelSet& L) {
 // with few items is scanned in one-warp Kogge-Stone chunks of 32 (shortest
 // chain of dependent combines).  An explicit radix folds that many items per
 // thread at every level.
-void default_shape(const sqsm_ctx* ctx, const int64_t* offsets, int64_t batch, int* L0, int* R) {
+void default_shape(const sqsm_ctx* ctx, int dtype, int nx, const int64_t* offsets, int64_t batch,
+                   int* L0, int* R) {
   const int64_t steps = offsets[batch] - offsets[0];
   *L0 = ctx->opt.leaf_chunk > 0 ? ctx->opt.leaf_chunk
         : steps <= 3 * int64_t(256) * ctx->sm_count ? 3 : 4;
   *R = ctx->opt.radix <= 1 ? 0 : ctx->opt.radix;
+  // FP64: a step per leaf thread costs its four kernels 64 cycles an
+  // instruction (two iterations with 1 / 2 / 3 steps: n = 4000 1.36 / 1.68 /
+  // 2.15 ms, 32000 2.97 / 2.55 / 2.82)
+  if (ctx->opt.leaf_chunk <= 0 && lane_plan(dtype, nx, *R))
+    *L0 = steps <= 8192 ? 1 : steps <= 32768 ? 2 : *L0;
 }
 
-Plan* find_plan(sqsm_ctx* ctx, const int64_t* offsets, int64_t batch, int L0, int R) {
+Plan* find_plan(sqsm_ctx* ctx, const int64_t* offsets, int64_t batch, int L0, int R, bool lanes) {
   for (auto& p : ctx->plans)
-    if (p->B == batch && p->L0 == L0 && p->R == R &&
+    if (p->B == batch && p->L0 == L0 && p->R == R && p->lanes == lanes &&
         std::memcmp(p->offsets.data(), offsets, sizeof(int64_t) * (batch + 1)) == 0)
       return p.get();
   return nullptr;
@@ -282,9 +313,10 @@ void drop_plan(sqsm_ctx* ctx, const Plan* victim) {
     }
 }
 
-Plan* get_plan(sqsm_ctx* ctx, const int64_t* offsets, int64_t batch, int L0, int R) {
-  if (Plan* q = find_plan(ctx, offsets, batch, L0, R)) return q;
+Plan* get_plan(sqsm_ctx* ctx, const int64_t* offsets, int64_t batch, int L0, int R, bool lanes) {
+  if (Plan* q = find_plan(ctx, offsets, batch, L0, R, lanes)) return q;
   auto p = std::make_unique<Plan>();
+  p->lanes = lanes;
   p->B = (int)batch;
   p->L0 = L0;
   p->R = R;
@@ -297,16 +329,18 @@ Plan* get_plan(sqsm_ctx* ctx, const int64_t* offsets, int64_t batch, int L0, int
     nf[b] = offsets[b + 1] - offsets[b];
     ns[b] = nf[b] + 1;
   }
-  if (!build_levels(*p, nf, p->filt) || !build_levels(*p, ns, p->smth)) return nullptr;
+  if (!build_levels(*p, nf, p->filt, ctx->sm_count, kLaneFilterChunk) ||
+      !build_levels(*p, ns, p->smth, ctx->sm_count, kLaneSmootherChunk))
+    return nullptr;
   if (ctx->plans.size() >= 8) drop_plan(ctx, ctx->plans.front().get());
   ctx->plans.push_back(std::move(p));
   return ctx->plans.back().get();
 }
 
-Plan* get_plan(sqsm_ctx* ctx, const int64_t* offsets, int64_t batch) {
+Plan* get_plan(sqsm_ctx* ctx, int dtype, int nx, const int64_t* offsets, int64_t batch) {
   int L0, R;
-  default_shape(ctx, offsets, batch, &L0, &R);
-  return get_plan(ctx, offsets, batch, L0, R);
+  default_shape(ctx, dtype, nx, offsets, batch, &L0, &R);
+  return get_plan(ctx, offsets, batch, L0, R, lane_plan(dtype, nx, R));
 }
 
 bool alloc_scan(Alloc& mem, const LevelSet& L, ScanBuffers& W, size_t item_bytes,
@@ -590,7 +624,7 @@ int sqsm_lgssm_smooth(sqsm_ctx* ctx, int dtype, int nx, int ny, int64_t n, const
     return fail(ctx, SQSM_ERR_INVALID_ARG, "pointer not a multiple of its element size");
   DeviceGuard g(ctx->device);
   const int64_t offsets[2] = {0, n};
-  Plan* p = get_plan(ctx, offsets, 1);
+  Plan* p = get_plan(ctx, dtype, nx, offsets, 1);
   if (!p) return fail(ctx, SQSM_ERR_NO_MEMORY, "plan allocation failed");
   Workspace* w = get_ws(p, dtype, nx);
   if (!w) return fail(ctx, SQSM_ERR_NO_MEMORY, "workspace allocation failed");
@@ -747,7 +781,7 @@ int choose_ipls_shape(sqsm_ctx* ctx, int dtype, const sqsm_model* model, const d
                       int lin, int64_t batch, const int64_t* offsets, const void* y,
                       const void* m0, const void* N0, const void* init_ms, const void* init_Ns,
                       void* ms, void* Ns, cudaStream_t s, int* L0, int* R) {
-  default_shape(ctx, offsets, batch, L0, R);
+  default_shape(ctx, dtype, 5, offsets, batch, L0, R);
   if (!ctx->opt.autotune || ctx->opt.leaf_chunk > 0 || ctx->opt.radix > 0) return SQSM_OK;
   const TuneKey key = tune_key(dtype, lin, batch, offsets);
   auto found = ctx->tuned.find(key);
@@ -766,8 +800,9 @@ int choose_ipls_shape(sqsm_ctx* ctx, int dtype, const sqsm_model* model, const d
   bool best_made = false;   // the best plan was made only for the measurement
   int rc = SQSM_OK;
   for (const auto& c : kTuneShapes) {
-    const bool existed = find_plan(ctx, offsets, batch, c[0], c[1]) != nullptr;
-    Plan* p = get_plan(ctx, offsets, batch, c[0], c[1]);
+    const bool lanes = lane_plan(dtype, 5, c[1]);
+    const bool existed = find_plan(ctx, offsets, batch, c[0], c[1], lanes) != nullptr;
+    Plan* p = get_plan(ctx, offsets, batch, c[0], c[1], lanes);
     if (!p) continue;
     Workspace* w = get_ws(p, dtype, 5);
     const void* n0 = w && ensure_ipls(w, p, dtype) &&
@@ -798,7 +833,7 @@ int choose_ipls_shape(sqsm_ctx* ctx, int dtype, const sqsm_model* model, const d
     }
     if (rc != SQSM_OK) break;
     if (t < best) {
-      if (best_made) drop_plan(ctx, find_plan(ctx, offsets, batch, bl, br));
+      if (best_made) drop_plan(ctx, find_plan(ctx, offsets, batch, bl, br, lane_plan(dtype, 5, br)));
       best = t;
       bl = c[0];
       br = c[1];
@@ -823,7 +858,7 @@ extern "C" int sqsm_scan_shape(sqsm_ctx* ctx, int dtype, int linearization, int6
   if (!ctx || !leaf_chunk || !radix) return SQSM_ERR_INVALID_ARG;
   if (batch < 1 || batch > (1 << 30) || !valid_offsets(offsets, batch))
     return fail(ctx, SQSM_ERR_INVALID_ARG, "offsets must start at 0 and increase strictly");
-  default_shape(ctx, offsets, batch, leaf_chunk, radix);
+  default_shape(ctx, dtype, 5, offsets, batch, leaf_chunk, radix);
   if (ctx->opt.autotune && ctx->opt.leaf_chunk <= 0 && ctx->opt.radix <= 0) {
     auto it = ctx->tuned.find(tune_key(dtype, linearization, batch, offsets));
     if (it != ctx->tuned.end()) {
@@ -865,15 +900,15 @@ int sqsm_ipls_smooth(sqsm_ctx* ctx, int dtype, const sqsm_model* model, const do
   cudaGetLastError();
   int L0 = 0, R = 0;
   if (pop) {
-    default_shape(ctx, offsets, batch, &L0, &R);
+    default_shape(ctx, dtype, 1, offsets, batch, &L0, &R);
   } else {
     const int trc = choose_ipls_shape(ctx, dtype, model, theta, linearization, batch, offsets, y,
                                       m0, N0, init_ms, init_Ns, ms, Ns, s, &L0, &R);
     if (trc != SQSM_OK) return trc;
   }
-  Plan* p = get_plan(ctx, offsets, batch, L0, R);
-  if (!p) return fail(ctx, SQSM_ERR_NO_MEMORY, "plan allocation failed");
   const int nx = pop ? 1 : 5, ny = pop ? 1 : 2;
+  Plan* p = get_plan(ctx, offsets, batch, L0, R, lane_plan(dtype, nx, R));
+  if (!p) return fail(ctx, SQSM_ERR_NO_MEMORY, "plan allocation failed");
   Workspace* w = get_ws(p, dtype, nx);
   if (!w || !ensure_ipls(w, p, dtype, nx, ny) ||
       (ctx->opt.refine > 0 && !ensure_refine_tabs(w, p, dtype, nx)))
@@ -980,15 +1015,15 @@ int sqsm_ipls_smooth_tol(sqsm_ctx* ctx, int dtype, const sqsm_model* model, cons
   cudaGetLastError();
   int L0 = 0, R = 0;
   if (pop) {
-    default_shape(ctx, offsets, batch, &L0, &R);
+    default_shape(ctx, dtype, 1, offsets, batch, &L0, &R);
   } else {
     const int trc = choose_ipls_shape(ctx, dtype, model, theta, linearization, batch, offsets, y,
                                       m0, N0, init_ms, init_Ns, ms, Ns, s, &L0, &R);
     if (trc != SQSM_OK) return trc;
   }
-  Plan* p = get_plan(ctx, offsets, batch, L0, R);
-  if (!p) return fail(ctx, SQSM_ERR_NO_MEMORY, "plan allocation failed");
   const int nx = pop ? 1 : 5, ny = pop ? 1 : 2;
+  Plan* p = get_plan(ctx, offsets, batch, L0, R, lane_plan(dtype, nx, R));
+  if (!p) return fail(ctx, SQSM_ERR_NO_MEMORY, "plan allocation failed");
   Workspace* w = get_ws(p, dtype, nx);
   if (!w || !ensure_ipls(w, p, dtype, nx, ny) ||
       (ctx->opt.refine > 0 && !ensure_refine_tabs(w, p, dtype, nx)))
@@ -1137,8 +1172,8 @@ int sqsm_ipls_smooth_std(sqsm_ctx* ctx, int dtype, const sqsm_model* model, cons
   cudaStream_t s = (cudaStream_t)stream;
   cudaGetLastError();
   int L0 = 0, R = 0;
-  default_shape(ctx, offsets, batch, &L0, &R);
-  Plan* p = get_plan(ctx, offsets, batch, L0, 4);   // fold-only levels
+  default_shape(ctx, SQSM_F32, 5, offsets, batch, &L0, &R);
+  Plan* p = get_plan(ctx, offsets, batch, L0, 4, false);   // fold-only levels
   if (!p) return fail(ctx, SQSM_ERR_NO_MEMORY, "plan allocation failed");
   Workspace* w = get_ws(p, dtype, 5);
   if (!w || !ensure_ipls(w, p, dtype)) return fail(ctx, SQSM_ERR_NO_MEMORY, "workspace");
@@ -1170,7 +1205,7 @@ static int nll_grad_run(sqsm_ctx* ctx, int dtype, const sqsm_model* model, const
   const int trc = choose_ipls_shape(ctx, dtype, model, theta, linearization, batch, offsets, y,
                                     m0, N0, init_ms, init_Ns, ms, Ns, s, &L0, &R);
   if (trc != SQSM_OK) return trc;
-  Plan* p = get_plan(ctx, offsets, batch, L0, R);
+  Plan* p = get_plan(ctx, offsets, batch, L0, R, lane_plan(dtype, 5, R));
   if (!p) return fail(ctx, SQSM_ERR_NO_MEMORY, "plan allocation failed");
   Workspace* w = get_ws(p, dtype, 5);
   if (!w || !ensure_ipls(w, p, dtype) || !ensure_adj(w, p, dtype) ||
@@ -1340,7 +1375,7 @@ int sqsm_ct_linearize(sqsm_ctx* ctx, int dtype, const sqsm_model* model, const d
   if (!aligned(elem_bytes(dtype), {y, ms, Ns, F, c, SQ, H, d, SR}))
     return fail(ctx, SQSM_ERR_INVALID_ARG, "pointer not a multiple of its element size");
   DeviceGuard g(ctx->device);
-  Plan* p = get_plan(ctx, offsets, batch);
+  Plan* p = get_plan(ctx, dtype, 5, offsets, batch);
   if (!p) return fail(ctx, SQSM_ERR_NO_MEMORY, "plan allocation failed");
   Workspace* w = get_ws(p, dtype, 5);
   if (!w || !ensure_ipls(w, p, dtype)) return fail(ctx, SQSM_ERR_NO_MEMORY, "workspace");

@@ -6,14 +6,29 @@
 #include <vector>
 
 #include "wscan.cuh"
+#include "lane_scan.cuh"
 #include "refine_filter.cuh"
 
 namespace sqsm {
+
+// Forms of a chunk level: sequential folds (one thread per chunk), one-warp
+// Kogge-Stone chunks of 32 items, and the two with a combine spread over
+// lanes (lane_scan.cuh): Kogge-Stone chunks of one block, sequential folds of
+// one 16-lane (smoother: 8-lane) group per chunk.  The lane forms hold in a
+// plan made for FP64 and n_x >= kLaneMinNx; another scan over that plan (the
+// adjoint's) takes a lane chunk as a chunk and a lane fold as a fold.
+enum LevelForm { kFoldLevel = 0, kChunkLevel, kLaneChunkLevel, kLaneFoldLevel };
+constexpr int kLaneMinNx = 3;
+
+template <typename T, int NX> constexpr bool lane_forms() {
+  return sizeof(T) == 8 && NX >= kLaneMinNx && NX <= kLaneRows;
+}
 
 // Levels of one scan (filter or smoother) for one batch layout.
 // lv[l] (l = 0..Lc-1) folds the items of level l into items[l+1];
 // n_items[l] is the number of items at level l (n_items[Lc] = B).
 struct LevelSet {
+  bool lanes = false;                  // upper levels in the lane forms
   std::vector<DevLevel> lv;
   std::vector<int64_t> n_items;
   int64_t* leaf_chunk_off = nullptr;   // device, B+1
@@ -22,10 +37,10 @@ struct LevelSet {
   std::vector<int64_t*> seq_item_off;
   std::vector<int64_t> max_seq_items;
   int B = 0;
-  // per chunk level l >= 1: 1 = one-warp Kogge-Stone chunks of 32 items,
-  // 0 = sequential folds (one thread per chunk)
+  // per chunk level l >= 1: how its chunks are scanned
   std::vector<char> cs;
-  bool chunk_scan(int l) const { return l < (int)cs.size() && cs[l]; }
+  char form(int l) const { return l < (int)cs.size() ? cs[l] : (char)kFoldLevel; }
+  bool chunk_scan(int l) const { return form(l) == kChunkLevel || form(l) == kLaneChunkLevel; }
 
   // Lowest item level whose per-sequence item count fits one Kogge-Stone block.
   int ks_level(int ks_max) const {
@@ -179,7 +194,8 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
   // and factors do not fit three such threads' registers.
   constexpr bool R3 = sizeof(T) == 4;
   constexpr int KS = R3 ? Ks3Max<T, FRec<NX>::size>::value : KsMax<T, FRec<NX>::size>::value;
-  const int Lk = L.ks_level(KS);
+  const bool lanes = lane_forms<T, NX>() && L.lanes;
+  const int Lk = L.ks_level(lanes ? kLaneFilterChunk : KS);
   const FMeansLayout fm = ftab ? fmeans_layout(L, sizeof(T), NX) : FMeansLayout{};
   const bool mo = means_only && fm.on;
   auto tab = [&](int l) {
@@ -200,6 +216,18 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
     }
     for (int l = 1; l < Lk; ++l) {
       ProfScope ps(P, K_FILTER_UP, s);
+      if constexpr (lane_forms<T, NX>()) {
+        if (L.form(l) == kLaneChunkLevel) {
+          filter_up_lane_ks<T, NX><<<(unsigned)L.lv[l].n_chunks, 2 * kLaneRows * kLaneFilterChunk,
+                                     0, s>>>(L.lv[l], (T*)W.items[l], (T*)W.items[l + 1]);
+          continue;
+        }
+        if (L.form(l) == kLaneFoldLevel) {
+          filter_up_lane<T, NX><<<(unsigned)((L.lv[l].n_chunks + 1) / 2), kWarp, 0, s>>>(
+              L.lv[l], (const T*)W.items[l], (T*)W.items[l + 1]);
+          continue;
+        }
+      }
       if constexpr (R3) {
         if (cs3_level(L, l, R3)) {
           const unsigned g = (unsigned)L.lv[l].n_chunks;
@@ -244,6 +272,13 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
       else
         filter_top_ks3<T, NX, false><<<L.B, 3 * KS, 0, s>>>(
             L.seq_item_off[Lk], (const T*)W.items[Lk], (T*)W.carry[Lk], W.flag[Lk], tab(Lk));
+    } else if constexpr (lane_forms<T, NX>()) {
+      if (lanes)
+        filter_top_lane_ks<T, NX><<<L.B, 2 * kLaneRows * kLaneFilterChunk, 0, s>>>(
+            L.seq_item_off[Lk], (const T*)W.items[Lk], (T*)W.carry[Lk], W.flag[Lk]);
+      else
+        filter_top_ks<T, NX><<<L.B, KS, 0, s>>>(L.seq_item_off[Lk], (const T*)W.items[Lk],
+                                                (T*)W.carry[Lk], W.flag[Lk]);
     } else
       filter_top_ks<T, NX><<<L.B, KS, 0, s>>>(L.seq_item_off[Lk], (const T*)W.items[Lk],
                                               (T*)W.carry[Lk], W.flag[Lk]);
@@ -252,6 +287,20 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
   }
   for (int l = (Lc > 1 ? Lk : Lc) - 1; l >= 1; --l) {
     ProfScope ps(P, K_FILTER_DOWN, s);
+    if constexpr (lane_forms<T, NX>()) {
+      if (L.form(l) == kLaneChunkLevel) {
+        filter_down_lane_ks<T, NX><<<(unsigned)L.lv[l].n_chunks, kLaneRows * kLaneFilterChunk, 0,
+                                     s>>>(L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1],
+                                          W.flag[l + 1], (T*)W.carry[l], W.flag[l]);
+        continue;
+      }
+      if (L.form(l) == kLaneFoldLevel) {
+        filter_down_lane<T, NX><<<(unsigned)((L.lv[l].n_chunks + 3) / 4), kWarp, 0, s>>>(
+            L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1], W.flag[l + 1],
+            (T*)W.carry[l], W.flag[l]);
+        continue;
+      }
+    }
     if (L.chunk_scan(l))
       filter_down_cs<T, NX><<<cs_down_grid(L.lv[l].n_chunks), kBlock, 0, s>>>(
           L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1], W.flag[l + 1],
@@ -276,7 +325,8 @@ void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv
                       unsigned* dmax = nullptr, T* etab = nullptr) {
   const int Lc = (int)L.lv.size();
   constexpr int KS = KsMax<T, SRec<NX>::size>::value;
-  const int Lk = L.ks_level(KS);
+  const bool lanes = lane_forms<T, NX>() && L.lanes;
+  const int Lk = L.ks_level(lanes ? kLaneSmootherChunk : KS);
   if (Lc > 1) {
     {
       ProfScope ps(P, K_SMOOTHER_LEAF_UP, s);
@@ -285,6 +335,18 @@ void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv
     }
     for (int l = 1; l < Lk; ++l) {
       ProfScope ps(P, K_SMOOTHER_UP, s);
+      if constexpr (lane_forms<T, NX>()) {
+        if (L.form(l) == kLaneChunkLevel) {
+          smoother_up_lane_ks<T, NX><<<(unsigned)L.lv[l].n_chunks, kLaneRows * kLaneSmootherChunk,
+                                       0, s>>>(L.lv[l], (T*)W.items[l], (T*)W.items[l + 1]);
+          continue;
+        }
+        if (L.form(l) == kLaneFoldLevel) {
+          smoother_up_lane<T, NX><<<(unsigned)((L.lv[l].n_chunks + 3) / 4), kWarp, 0, s>>>(
+              L.lv[l], (const T*)W.items[l], (T*)W.items[l + 1]);
+          continue;
+        }
+      }
       if (L.chunk_scan(l))
         smoother_up_cs<T, NX><<<(unsigned)L.lv[l].n_chunks, kChunkScan, 0, s>>>(
             L.lv[l], (T*)W.items[l], (T*)W.items[l + 1]);
@@ -296,14 +358,37 @@ void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv
             L.lv[l], (const T*)W.items[l], (T*)W.items[l + 1]);
     }
     ProfScope ps(P, K_SMOOTHER_UP, s);
-    smoother_top_ks<T, NX><<<L.B, KS, 0, s>>>(L.seq_item_off[Lk],
-                                                          (const T*)W.items[Lk], (T*)W.carry[Lk],
-                                                          W.flag[Lk]);
+    bool top = false;
+    if constexpr (lane_forms<T, NX>()) {
+      if (lanes) {
+        smoother_top_lane_ks<T, NX><<<L.B, kLaneRows * kLaneSmootherChunk, 0, s>>>(
+            L.seq_item_off[Lk], (const T*)W.items[Lk], (T*)W.carry[Lk], W.flag[Lk]);
+        top = true;
+      }
+    }
+    if (!top)
+      smoother_top_ks<T, NX><<<L.B, KS, 0, s>>>(L.seq_item_off[Lk], (const T*)W.items[Lk],
+                                                (T*)W.carry[Lk], W.flag[Lk]);
   } else {
     cudaMemsetAsync(W.flag[Lc], 0, sizeof(int) * L.n_items[Lc], s);
   }
   for (int l = (Lc > 1 ? Lk : Lc) - 1; l >= 1; --l) {
     ProfScope ps(P, K_SMOOTHER_DOWN, s);
+    if constexpr (lane_forms<T, NX>()) {
+      if (L.form(l) == kLaneChunkLevel) {
+        smoother_down_lane_ks<T, NX><<<(unsigned)L.lv[l].n_chunks, kLaneRows * kLaneSmootherChunk,
+                                       0, s>>>(L.lv[l], (const T*)W.items[l],
+                                               (const T*)W.carry[l + 1], W.flag[l + 1],
+                                               (T*)W.carry[l], W.flag[l]);
+        continue;
+      }
+      if (L.form(l) == kLaneFoldLevel) {
+        smoother_down_lane<T, NX><<<(unsigned)((L.lv[l].n_chunks + 3) / 4), kWarp, 0, s>>>(
+            L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1], W.flag[l + 1],
+            (T*)W.carry[l], W.flag[l]);
+        continue;
+      }
+    }
     if (L.chunk_scan(l))
       smoother_down_cs<T, NX><<<cs_down_grid(L.lv[l].n_chunks), kBlock, 0, s>>>(
           L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1], W.flag[l + 1],
