@@ -71,7 +71,7 @@ void adj_enqueue(const IplsArgs& a, const AdjArgs& g, const LevelSet& Lf, const 
   enqueue_filter<T, NX, NY>(Lf, Wf, sq, gv, (const T*)a.y, (const T*)a.m0, (const T*)a.N0, fo,
                             partial, status, s);
   enqueue_smoother<T, NX, NY>(Ls, Ws, sq, gv, fo, so, status, s);
-  enqueue_loglik_reduce(sq, partial, g.ll, status, s);
+  enqueue_loglik_reduce(sq, partial, Lf.max_seq_items[1], g.ll, status, s);
   adj_nll_kernel<<<1, 1, 0, s>>>(sq.B, g.ll, -1.0, g.nll);
   // how far n* is from a fixed point of Alg. 3: the relative change of the
   // smoothing means in that one more iteration (words 2, 3)

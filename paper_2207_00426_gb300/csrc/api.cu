@@ -648,7 +648,7 @@ int sqsm_lgssm_smooth(sqsm_ctx* ctx, int dtype, int nx, int ny, int64_t n, const
                : lgssm_enqueue_f64(a, p->filt, w->filt, p->smth, w->smth, sq, w->partial,
                                    ctx->d_status, s);
   if (rc) return fail(ctx, rc, "(nx, ny) pair not compiled in");
-  if (loglik) enqueue_loglik_reduce(sq, w->partial, loglik, ctx->d_status, s, prof);
+  if (loglik) enqueue_loglik_reduce(sq, w->partial, p->filt.max_seq_items[1], loglik, ctx->d_status, s, prof);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "sqsm_lgssm_smooth launch");
   return SQSM_OK;

@@ -125,8 +125,10 @@ void adj_enqueue_f64(const IplsArgs& a, const AdjArgs& g, const LevelSet& Lf,
 void ct_linearize_f32(const IplsArgs& a, const LevelSet& Lf, DevSeqs sq, cudaStream_t s);
 void ct_linearize_f64(const IplsArgs& a, const LevelSet& Lf, DevSeqs sq, cudaStream_t s);
 
-void enqueue_loglik_reduce(DevSeqs sq, const double* partial, double* loglik, int* status,
-                           cudaStream_t s, Prof* P = nullptr);
+// Log-likelihood of every sequence from its leaf chunks' partial sums (which
+// it may overwrite); max_chunks: the most chunks any sequence has.
+void enqueue_loglik_reduce(DevSeqs sq, double* partial, int64_t max_chunks, double* loglik,
+                           int* status, cudaStream_t s, Prof* P = nullptr);
 
 // Largest state dimension of the prior Cholesky kernel.
 constexpr int kMaxPriorNx = 8;

@@ -48,7 +48,7 @@ void ipls_phase_model(const IplsArgs& a, const LevelSet& Lf, const ScanBuffers& 
     ProfScope ps(a.prof, K_INIT, s);
     if (a.init_ms) {
       const RowsSplit<T, NX> init{(T*)a.init_ms, (T*)a.init_Ns};
-      rows_copy_kernel<T, NX><<<grid_for(rows), kBlock, 0, s>>>(rows, init, nom);
+      rows_convert_kernel<T, NX, true><<<grid_for(rows), kBlock, 0, s>>>(rows, init, nom);
     } else {
       broadcast_prior_kernel<T, NX><<<grid_for(Ls.lv[0].n_chunks), kBlock, 0, s>>>(
           Ls.lv[0], (const T*)a.m0, (const T*)a.N0, nom);
@@ -59,9 +59,9 @@ void ipls_phase_model(const IplsArgs& a, const LevelSet& Lf, const ScanBuffers& 
     {
       ProfScope ps(a.prof, K_INIT, s);
       const RowsSplit<T, NX> user{(T*)a.ms, (T*)a.Ns};
-      rows_copy_kernel<T, NX><<<grid_for(rows), kBlock, 0, s>>>(rows, nom, user);
+      rows_convert_kernel<T, NX, false><<<grid_for(rows), kBlock, 0, s>>>(rows, user, nom);
     }
-    if (a.loglik) enqueue_loglik_reduce(sq, partial, a.loglik, status, s, a.prof);
+    if (a.loglik) enqueue_loglik_reduce(sq, partial, Lf.max_seq_items[1], a.loglik, status, s, a.prof);
     return;
   }
   // the linearised model of every step, packed (a.F holds the PRec records)

@@ -5,29 +5,57 @@ namespace sqsm {
 
 // One block per sequence: strided FP64 partial sums, then a fixed-order
 // shared-memory tree, so the result does not depend on scheduling.
-__global__ void loglik_reduce(DevSeqs sq, const double* __restrict__ partial,
-                              double* __restrict__ loglik, int* status) {
+// Sum of part[lo], part[lo + stride], ... below hi by a block of 256 threads,
+// in a fixed order (valid in thread 0).
+__device__ double block_sum(const double* part, int64_t lo, int64_t hi, int64_t stride) {
   __shared__ double buf[256];
-  const int b = blockIdx.x;
-  const int64_t lo = sq.leaf_chunk_off[b], hi = sq.leaf_chunk_off[b + 1];
   double acc = 0.0;
-  for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) acc += partial[i];
+  for (int64_t i = lo + threadIdx.x * stride; i < hi; i += blockDim.x * stride) acc += part[i];
   buf[threadIdx.x] = acc;
   __syncthreads();
   for (int w = blockDim.x / 2; w > 0; w >>= 1) {
     if (threadIdx.x < w) buf[threadIdx.x] += buf[threadIdx.x + w];
     __syncthreads();
   }
+  return buf[0];
+}
+
+__global__ void loglik_reduce(DevSeqs sq, const double* __restrict__ partial, int64_t stride,
+                              double* __restrict__ loglik, int* status) {
+  const int b = blockIdx.x;
+  const double v = block_sum(partial, sq.leaf_chunk_off[b], sq.leaf_chunk_off[b + 1], stride);
   if (threadIdx.x == 0) {
-    loglik[b] = buf[0];
-    if (!isfinite(buf[0]) && status) atomicOr(status, 8);
+    loglik[b] = v;
+    if (!isfinite(v) && status) atomicOr(status, 8);
   }
 }
 
-void enqueue_loglik_reduce(DevSeqs sq, const double* partial, double* loglik, int* status,
-                           cudaStream_t s, Prof* P) {
+// First stage for long sequences: block (slice, sequence) puts the sum of its
+// slice in the slice's first entry.
+__global__ void loglik_slices(DevSeqs sq, double* partial, int64_t slice) {
+  const int b = blockIdx.y;
+  const int64_t hi = sq.leaf_chunk_off[b + 1], lo = sq.leaf_chunk_off[b] + blockIdx.x * slice;
+  if (lo >= hi) return;
+  const double v = block_sum(partial, lo, lo + slice < hi ? lo + slice : hi, 1);
+  if (threadIdx.x == 0) partial[lo] = v;
+}
+
+// One SM adds a warp of doubles in 19 cycles, so a block per sequence took
+// 13 us for the 33334 chunks of n = 1e5; sequences of more than a slice are
+// summed in slices by many blocks first (7 us, both launches).
+constexpr int64_t kLoglikSlice = 2048;
+
+void enqueue_loglik_reduce(DevSeqs sq, double* partial, int64_t max_chunks, double* loglik,
+                           int* status, cudaStream_t s, Prof* P) {
   ProfScope ps(P, K_LOGLIK, s);
-  loglik_reduce<<<sq.B, 256, 0, s>>>(sq, partial, loglik, status);
+  const int64_t slices = (max_chunks + kLoglikSlice - 1) / kLoglikSlice;
+  // (a grid's second dimension holds 65535 blocks)
+  const bool sliced = slices > 1 && sq.B <= 65535;
+  if (sliced) {
+    loglik_slices<<<dim3((unsigned)slices, (unsigned)sq.B), 256, 0, s>>>(sq, partial,
+                                                                          kLoglikSlice);
+  }
+  loglik_reduce<<<sq.B, 256, 0, s>>>(sq, partial, sliced ? kLoglikSlice : 1, loglik, status);
 }
 
 namespace {

@@ -276,7 +276,7 @@ extern "C" int sqsm_lgssm_smooth_noalloc(int dtype, int nx, int ny, int64_t n, c
                        ? lgssm_enqueue_f32(a, Lf, Wf, Ls, Ws, sq, partial, nullptr, s)
                        : lgssm_enqueue_f64(a, Lf, Wf, Ls, Ws, sq, partial, nullptr, s);
     if (rc) return rc;
-    if (loglik) enqueue_loglik_reduce(sq, partial, loglik, nullptr, s);
+    if (loglik) enqueue_loglik_reduce(sq, partial, Lf.lv[0].n_chunks, loglik, nullptr, s);
     if (cudaGetLastError() != cudaSuccess) return SQSM_ERR_CUDA;
   }
   return SQSM_OK;

@@ -367,9 +367,4 @@ smoother_leaf_down(DevLevel lv, DevSeqs sq, GV gv, FO fo, const T* __restrict__ 
   }
 }
 
-// Per-sequence FP64 sum of the leaf partial log-likelihoods in a fixed
-// order (deterministic).  One block per sequence.
-__global__ void loglik_reduce(DevSeqs sq, const double* __restrict__ partial,
-                              double* __restrict__ loglik, int* status);
-
 }  // namespace sqsm

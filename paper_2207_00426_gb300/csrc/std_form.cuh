@@ -948,7 +948,7 @@ void std_ipls_enqueue(const IplsArgs& a, const LevelSet& Lf, const ScanBuffers& 
   }
   const RowsSplitSym<T, NX> user{(T*)a.ms, (T*)a.Ns};
   rows_copy_kernel<T, NX><<<grid_for(rows), kBlock, 0, s>>>(rows, nom, user);
-  if (a.loglik) enqueue_loglik_reduce(sq, partial, a.loglik, status, s, nullptr);
+  if (a.loglik) enqueue_loglik_reduce(sq, partial, Lf.max_seq_items[1], a.loglik, status, s, nullptr);
 }
 
 }  // namespace sqsm

@@ -1,4 +1,6 @@
-"""The Gauss-Hermite regression with 16 lanes per step."""
+"""Small launches of the smoothers' bookkeeping at the sizes where they change:
+conversion of state rows (blocks of 128), the log-likelihood's sum in slices
+of 2048 chunks, the Gauss-Hermite regression with 16 lanes per step."""
 import numpy as np
 import pytest
 
@@ -16,6 +18,38 @@ def B():
 
 def _t(a, dt):
     return torch.tensor(np.ascontiguousarray(a), dtype=dt, device="cuda:0")
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.float64])
+@pytest.mark.parametrize("lengths", [[1], [126], [127], [128], [255, 1, 3]])
+def test_rows_conversion_is_exact(B, dt, lengths):
+    """Two iterations equal one iteration and another from its result, bit for
+    bit: the caller's rows and the packed ones hold the same numbers."""
+    d = W.ct_batch(batch=len(lengths), lengths=lengths, seed=5)
+    ctx = B.Context(0)
+    a = (ctx, d["theta"], _t(d["y"], dt), d["offsets"], _t(d["m0"], dt), _t(d["N0"], dt))
+    two = B.sqsm_ipls_smooth(*a, 2)
+    one = B.sqsm_ipls_smooth(*a, 1)
+    junk = one[1] + torch.triu(torch.ones(5, 5, dtype=dt, device="cuda:0"), 1)   # ignored part
+    again = B.sqsm_ipls_smooth(*a, 1, init_ms=one[0], init_Ns=junk)
+    torch.cuda.synchronize()
+    for u, v in zip(two, again):
+        assert torch.equal(u, v)
+    assert torch.equal(two[1], torch.tril(two[1]))
+
+
+@pytest.mark.parametrize("n", [2048, 2049, 6145, 16384])
+def test_loglik_in_slices(B, n):
+    """One step per leaf: the sum of n partial values in slices of 2048 against
+    one chunk per sequence (a single running FP64 sum): both round each of
+    their n additions, so they differ by at most 2 n u of the absolute sum."""
+    m = W.linear_cv(n=n, seed=3)
+    q = {k: _t(v, torch.float64) for k, v in m.items() if k != "x"}
+    ll = [B.sqsm_lgssm_smooth(c, q["F"], q["c"], q["SQ"], q["H"], q["d"], q["SR"], q["m0"],
+                              q["N0"], q["y"])[4].item()
+          for c in (B.Context(0, leaf_chunk=1), B.Context(0, leaf_chunk=n))]
+    # every step's term is below 20 in magnitude here; recursion rounding 1e-10
+    assert abs(ll[0] - ll[1]) <= 2 * n * 2.0 ** -53 * 20 * n + 1e-10 * abs(ll[1])
 
 
 @pytest.mark.parametrize("lengths", [[1], [7], [8], [9, 1, 30], [200]])
