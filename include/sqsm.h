@@ -117,9 +117,11 @@ typedef struct {
 } sqsm_model;
 
 /* Scan shape.  Zero fields take defaults: leaf_chunk 3 when all leaf chunks
- * of a call fit one wave of 256 threads per SM, else 4; radix 0 folds upper
- * levels of more than 160000 items 4 per thread and scans smaller levels in
- * one-warp chunks of 32.
+ * of a call fit one wave of 256 threads per SM, else 4 (FP64 with n_x >= 3: 1
+ * up to 16384 time steps per call, 2 up to 65536; n_x < 3: 1 to 3 up to 12288
+ * steps); radix 0 folds upper levels of more than 160000 items 4 per thread
+ * and scans smaller levels in one-warp chunks of 32 (FP64 with n_x >= 3: in
+ * chunks and folds of few items, each combine spread over lanes).
  *
  * autotune = 1 (with leaf_chunk = radix = 0): the first sqsm_ipls_smooth or
  * sqsm_ipls_nll_grad call of each workload shape (dtype, linearisation,

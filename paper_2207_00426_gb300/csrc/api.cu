@@ -158,11 +158,12 @@ constexpr int64_t kFoldAboveItems = 160000;
 // thread, whose instructions then fill enough warps to keep every FP64 unit
 // busy (160 warps, one per SM); one with fewer is folded 4 per lane group,
 // whose combine issues a fifth of the instructions per warp but uses a
-// sixteenth of the warp; one that fits one block of Kogge-Stone chunks per
-// SM is scanned in such chunks.  Two iterations with one step per leaf,
-// n = 16000: 1.94 ms against 2.36 folded per thread; at n = 1e5 the two forms
-// are even.
+// sixteenth of the warp (n = 16000, one step per leaf, two iterations: 1.94 ms
+// against 2.36 folded per thread; at 100000 steps the two are even); one of
+// at most 32 items per SM is scanned in Kogge-Stone chunks (n = 2000: 1.15 ms
+// against 1.28 with a lane fold first, n = 12000: 1.68 against 1.75).
 constexpr int64_t kLaneMaxItems = 20000;
+constexpr int64_t kLaneChunkItemsPerSm = 32;
 
 // Levels of a segmented scan whose level-0 items are `counts[b]` per
 // sequence: chunks of L0 items at the leaf, then chunks of R items (or, for
@@ -186,9 +187,9 @@ bool build_levels(Plan& p, const std::vector<int64_t>& counts0, LevelSet& L, int
         int64_t items = 0;
         for (int64_t v : counts) items += v;
         if (p.lanes)
-          form = items > kLaneMaxItems                      ? kFoldLevel
-                 : items > int64_t(sm_count) * lane_chunk   ? kLaneFoldLevel
-                                                            : kLaneChunkLevel;
+          form = items > kLaneMaxItems                   ? kFoldLevel
+                 : items > kLaneChunkItemsPerSm * sm_count ? kLaneFoldLevel
+                                                           : kLaneChunkLevel;
         else
           form = items <= kFoldAboveItems ? kChunkLevel : kFoldLevel;
         size = form == kChunkLevel ? kChunkScan
@@ -265,25 +266,37 @@ bool lane_plan(int dtype, int nx, int R) {
   return dtype == SQSM_F64 && nx >= kLaneMinNx && R == 0;
 }
 
-// Scan shape from the options, else the default: leaf 3 steps per thread
-// while the leaf chunks fit one wave of the leaf kernels (256 threads per SM
-// at their register use), so that the latency-bound leaf chains are short, 4
-// above that (fewer upper items); radix 0: a level with many items is folded
-// 4 items per thread (enough threads to fill the GPU, least work), a level
-// with few items is scanned in one-warp Kogge-Stone chunks of 32 (shortest
-// chain of dependent combines).  An explicit radix folds that many items per
-// thread at every level.
+// Scan shape from the options, else the default.
+// Leaf: every step a leaf thread folds lengthens the four leaf kernels'
+// serial chains, every level above costs a launch and its combines.  FP32
+// takes 3 steps per thread while the leaf chunks fit one wave of the leaf
+// kernels (256 threads per SM at their register use), 4 above that (fewer
+// upper items).  In FP64 with the lane forms a step costs a leaf thread's four
+// kernels 64 cycles an instruction, and it takes one up to 16384 steps and two
+// up to 65536 (two iterations with 1 / 2 / 3 steps per leaf: n = 4000 1.36 /
+// 1.68 / 2.15 ms, 16000 1.94 / 2.01 / 2.45, 32000 2.97 / 2.55 / 2.82, 100000
+// 6.50 / 5.39 / 5.28).  (One step is faster in FP32 too, n = 1000 0.80 against
+// 1.01 ms per ten iterations, but its factors come out less exact in one
+// short track of ten: another bracketing is another draw of the rounding.)
+// With n_x < 3 a combine costs less than a launch: the leaf grows to three
+// steps where that leaves one chunk level and the top (4096 items).
+// radix 0: a level with many items is folded 4 items per thread (enough
+// threads to fill the GPU, least work), a level with few items is scanned in
+// one-warp Kogge-Stone chunks of 32 (shortest chain of dependent combines).
+// An explicit radix folds that many items per thread at every level.
 void default_shape(const sqsm_ctx* ctx, int dtype, int nx, const int64_t* offsets, int64_t batch,
                    int* L0, int* R) {
   const int64_t steps = offsets[batch] - offsets[0];
-  *L0 = ctx->opt.leaf_chunk > 0 ? ctx->opt.leaf_chunk
-        : steps <= 3 * int64_t(256) * ctx->sm_count ? 3 : 4;
   *R = ctx->opt.radix <= 1 ? 0 : ctx->opt.radix;
-  // FP64: a step per leaf thread costs its four kernels 64 cycles an
-  // instruction (two iterations with 1 / 2 / 3 steps: n = 4000 1.36 / 1.68 /
-  // 2.15 ms, 32000 2.97 / 2.55 / 2.82)
-  if (ctx->opt.leaf_chunk <= 0 && lane_plan(dtype, nx, *R))
-    *L0 = steps <= 8192 ? 1 : steps <= 32768 ? 2 : *L0;
+  if (ctx->opt.leaf_chunk > 0) {
+    *L0 = ctx->opt.leaf_chunk;
+    return;
+  }
+  *L0 = steps <= 3 * int64_t(256) * ctx->sm_count ? 3 : 4;
+  if (*R != 0) return;
+  const int64_t two_levels = (steps + 4095) / 4096;
+  if (nx < kLaneMinNx && two_levels <= 3) *L0 = (int)two_levels;
+  else if (lane_plan(dtype, nx, *R)) *L0 = steps <= 16384 ? 1 : steps <= 65536 ? 2 : *L0;
 }
 
 Plan* find_plan(sqsm_ctx* ctx, const int64_t* offsets, int64_t batch, int L0, int R, bool lanes) {

@@ -191,8 +191,10 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
                     bool means_only = false) {
   const int Lc = (int)L.lv.size();
   // FP32 takes three threads per combine at the top of the tree; FP64 records
-  // and factors do not fit three such threads' registers.
-  constexpr bool R3 = sizeof(T) == 4;
+  // and factors do not fit three such threads' registers, and below n_x = 3
+  // a combine is too short to be worth three (population model, n = 10000:
+  // 0.635 against 0.616 ms per 20 iterations with one).
+  constexpr bool R3 = sizeof(T) == 4 && NX >= kLaneMinNx;
   constexpr int KS = R3 ? Ks3Max<T, FRec<NX>::size>::value : KsMax<T, FRec<NX>::size>::value;
   const bool lanes = lane_forms<T, NX>() && L.lanes;
   const int Lk = L.ks_level(lanes ? kLaneFilterChunk : KS);

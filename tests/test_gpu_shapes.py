@@ -1,6 +1,7 @@
 """Small launches of the smoothers' bookkeeping at the sizes where they change:
 conversion of state rows (blocks of 128), the log-likelihood's sum in slices
-of 2048 chunks, the Gauss-Hermite regression with 16 lanes per step."""
+of 2048 chunks, the default leaf at the lengths where it changes, the
+Gauss-Hermite regression with 16 lanes per step."""
 import numpy as np
 import pytest
 
@@ -50,6 +51,26 @@ def test_loglik_in_slices(B, n):
           for c in (B.Context(0, leaf_chunk=1), B.Context(0, leaf_chunk=n))]
     # every step's term is below 20 in magnitude here; recursion rounding 1e-10
     assert abs(ll[0] - ll[1]) <= 2 * n * 2.0 ** -53 * 20 * n + 1e-10 * abs(ll[1])
+
+
+@pytest.mark.parametrize("nx,dt,n,leaf", [
+    (5, torch.float32, 1, 3), (5, torch.float32, 116_736, 3), (5, torch.float32, 116_737, 4),
+    (5, torch.float64, 1, 1), (5, torch.float64, 16_384, 1), (5, torch.float64, 16_385, 2),
+    (5, torch.float64, 65_536, 2), (5, torch.float64, 65_537, 3),
+    (1, torch.float32, 4096, 1), (1, torch.float32, 4097, 2), (1, torch.float32, 12_289, 3)])
+def test_default_leaf(B, nx, dt, n, leaf):
+    """The default context gives the bits of one with the leaf spelt out."""
+    if nx == 5:
+        if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+            assert B.Context(0).scan_shape([0, n], dt) == (leaf, 0)
+        return
+    d = W.ricker_batch([n], seed=3)
+    r = [B.sqsm_ipls_smooth_population(c, d["theta"], _t(d["y"], dt), d["offsets"],
+                                       _t(d["m0"], dt), _t(d["N0"], dt), 2)
+         for c in (B.Context(0), B.Context(0, leaf_chunk=leaf))]
+    torch.cuda.synchronize()
+    for u, v in zip(*r):
+        assert torch.equal(u, v)
 
 
 @pytest.mark.parametrize("lengths", [[1], [7], [8], [9, 1, 30], [200]])
