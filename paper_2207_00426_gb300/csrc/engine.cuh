@@ -171,6 +171,16 @@ inline FMeansLayout fmeans_layout(const LevelSet& L, size_t es, int nx) {
   return f;
 }
 
+// Level 1's down-sweep and the leaf's in one launch (filter_down_leaf): for
+// chunk-scanned levels of at most kFuseMaxItems items whose chunks leave at
+// most a fifth of the lanes idle.
+constexpr int64_t kFuseMaxItems = 65536;
+
+inline bool fuse_down(const LevelSet& L, int Lk) {
+  return Lk > 1 && L.form(1) == kChunkLevel && L.n_items[1] <= kFuseMaxItems &&
+         4 * kChunkScan * L.lv[1].n_chunks <= 5 * L.n_items[1] + 4 * kChunkScan;
+}
+
 // Allow a kernel the dynamic shared memory of its next launch where that
 // exceeds the 48 KB default (a function attribute, not a stream operation,
 // so it may be set while the stream is being captured).
@@ -287,7 +297,8 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
   } else {
     cudaMemsetAsync(W.flag[Lc], 0, sizeof(int) * L.n_items[Lc], s);
   }
-  for (int l = (Lc > 1 ? Lk : Lc) - 1; l >= 1; --l) {
+  const bool fused = Lc > 1 && fuse_down(L, Lk);
+  for (int l = (Lc > 1 ? Lk : Lc) - 1; l >= (fused ? 2 : 1); --l) {
     ProfScope ps(P, K_FILTER_DOWN, s);
     if constexpr (lane_forms<T, NX>()) {
       if (L.form(l) == kLaneChunkLevel) {
@@ -317,14 +328,19 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
           (T*)W.carry[l], W.flag[l]);
   }
   ProfScope ps(P, K_FILTER_LEAF_DOWN, s);
-  filter_leaf_down<T, NX, NY, GV, FO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
+  if (fused)
+    filter_down_leaf<T, NX, NY, GV, FO><<<cs_down_grid(L.lv[1].n_chunks), kBlock, 0, s>>>(
+        L.lv[1], (const T*)W.items[1], (const T*)W.carry[2], W.flag[2], L.lv[0], sq, gv, y, m0, N0,
+        fo, partial, status);
+  else
+    filter_leaf_down<T, NX, NY, GV, FO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
       L.lv[0], sq, gv, y, m0, N0, (const T*)W.carry[1], W.flag[1], fo, partial, status);
 }
 
 template <typename T, int NX, int NY, typename GV, typename FO, typename SO>
 void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv, FO fo, SO so,
                       int* status, cudaStream_t s, Prof* P = nullptr, bool add_nominal = false,
-                      unsigned* dmax = nullptr, T* etab = nullptr) {
+                      unsigned* dmax = nullptr, T* etab = nullptr, PriorMean<T> pm = {}) {
   const int Lc = (int)L.lv.size();
   constexpr int KS = KsMax<T, SRec<NX>::size>::value;
   const bool lanes = lane_forms<T, NX>() && L.lanes;
@@ -374,7 +390,8 @@ void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv
   } else {
     cudaMemsetAsync(W.flag[Lc], 0, sizeof(int) * L.n_items[Lc], s);
   }
-  for (int l = (Lc > 1 ? Lk : Lc) - 1; l >= 1; --l) {
+  const bool fused = Lc > 1 && fuse_down(L, Lk);
+  for (int l = (Lc > 1 ? Lk : Lc) - 1; l >= (fused ? 2 : 1); --l) {
     ProfScope ps(P, K_SMOOTHER_DOWN, s);
     if constexpr (lane_forms<T, NX>()) {
       if (L.form(l) == kLaneChunkLevel) {
@@ -405,8 +422,13 @@ void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv
           (T*)W.carry[l], W.flag[l]);
   }
   ProfScope ps(P, K_SMOOTHER_LEAF_DOWN, s);
-  smoother_leaf_down<T, NX, NY, GV, FO, SO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
-      L.lv[0], sq, gv, fo, (const T*)W.carry[1], W.flag[1], so, status, add_nominal, dmax);
+  if (fused)
+    smoother_down_leaf<T, NX, NY, GV, FO, SO><<<cs_down_grid(L.lv[1].n_chunks), kBlock, 0, s>>>(
+        L.lv[1], (const T*)W.items[1], (const T*)W.carry[2], W.flag[2], L.lv[0], sq, gv, fo, so,
+        status, add_nominal, dmax, pm);
+  else
+    smoother_leaf_down<T, NX, NY, GV, FO, SO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
+        L.lv[0], sq, gv, fo, (const T*)W.carry[1], W.flag[1], so, status, add_nominal, dmax, pm);
 }
 
 // Record sizes (elements) of the scan buffers.

@@ -53,6 +53,9 @@ void ipls_phase_model(const IplsArgs& a, const LevelSet& Lf, const ScanBuffers& 
       broadcast_prior_kernel<T, NX><<<grid_for(Ls.lv[0].n_chunks), kBlock, 0, s>>>(
           Ls.lv[0], (const T*)a.m0, (const T*)a.N0, nom);
     }
+    if (a.centered)
+      center_prior_kernel<T, NX><<<(sq.B + 127) / 128, 128, 0, s>>>(sq, (const T*)a.m0, nom,
+                                                                     (T*)a.dm0);
     return;
   }
   if (phase == IPLS_POST) {
@@ -75,11 +78,9 @@ void ipls_phase_model(const IplsArgs& a, const LevelSet& Lf, const ScanBuffers& 
     ProfScope ps(a.prof, K_SLR, s);
     slr(nom, s);
   }
-  if (a.centered) {
-    ProfScope ps(a.prof, K_INIT, s);
-    center_prior_kernel<T, NX><<<(sq.B + 127) / 128, 128, 0, s>>>(sq, (const T*)a.m0, nom,
-                                                                   (T*)a.dm0);
-  }
+  // (dm0 holds m0 - m_0: written with the initial trajectory, then by every
+  // smoother pass that moves m_0)
+  const PriorMean<T> pm{(const T*)a.m0, a.centered ? (T*)a.dm0 : nullptr};
   // refinement passes need the nominal rows from before each smoother pass
   const int passes = a.centered ? a.refine : 0;
   const RowsPacked<T, NX> prev{(T*)a.prevrows};
@@ -98,7 +99,7 @@ void ipls_phase_model(const IplsArgs& a, const LevelSet& Lf, const ScanBuffers& 
   // with refinement passes to follow, the first pass keeps each row's E_k
   T* etab = passes > 0 ? (T*)a.etab : nullptr;
   enqueue_smoother<T, NX, NY>(Ls, Ws, sq, gv, fr, nom, status, s, a.prof, a.centered != 0, dmax,
-                              etab);
+                              etab, pm);
   // Mixed-precision iterative refinement: the smoother's FP32 error is that
   // of a linear solve, so one more pass on the residual model about its own
   // result (offsets formed beyond FP32 precision) removes most of it; the
@@ -112,15 +113,14 @@ void ipls_phase_model(const IplsArgs& a, const LevelSet& Lf, const ScanBuffers& 
       ProfScope ps(a.prof, K_INIT, s);
       refine_residual_kernel<T, NX, NY><<<grid_for(Lf.lv[0].n_chunks * a.leaf), kBlock, 0, s>>>(
           Lf.lv[0], a.leaf, prev, nom, (T*)a.F);
-      center_prior_kernel<T, NX><<<(sq.B + 127) / 128, 128, 0, s>>>(sq, (const T*)a.m0, nom,
-                                                                     (T*)a.dm0);
     }
     if (r + 1 < passes) keep_prev();
     enqueue_filter<T, NX, NY>(Lf, Wf, sq, gv, (const T*)a.y, (const T*)a.dm0, (const T*)a.N0, fr,
                               a.partial2, status, s, a.prof, ftab, true);
     if (!etab || !enqueue_smoother_means<T, NX, NY>(Ls, Ws, sq, gv, fr, nom, etab, status, s,
-                                                    a.prof))
-      enqueue_smoother<T, NX, NY>(Ls, Ws, sq, gv, fr, nom, status, s, a.prof, true, nullptr);
+                                                    a.prof, pm))
+      enqueue_smoother<T, NX, NY>(Ls, Ws, sq, gv, fr, nom, status, s, a.prof, true, nullptr,
+                                  nullptr, pm);
   }
 }
 

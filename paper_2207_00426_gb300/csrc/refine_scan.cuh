@@ -134,29 +134,14 @@ smoother_top_ks_g(const int64_t* __restrict__ seq_item_off, const T* __restrict_
   }
 }
 
-// Chunk down-sweep (see smoother_down_cs), g only: each item's carry g.
+// As smoother_item_carry, g only.
 template <typename T, int NX>
-__global__ void __launch_bounds__(kBlock)
-smoother_down_cs_g(DevLevel lv, const T* __restrict__ items, const T* __restrict__ carry_in,
-                   const int* __restrict__ flag_in, T* __restrict__ carry_out,
-                   int* __restrict__ flag_out) {
+SQSM_DEV bool smoother_item_carry_g(const T* __restrict__ items, const T* __restrict__ carry_in,
+                                    int flag, int64_t c, int64_t i, int j, int cnt, bool active,
+                                    T* cg) {
   using R = SRec<NX>;
-  constexpr int REC = R::size, XS = XRow<NX>::size, W = (R::g + NX + 3) / 4 * 4;
-  static_assert(kChunkScan == kWarp && kBlock % kWarp == 0, "one chunk per warp");
-  __shared__ __align__(16) T SO[kBlock / kWarp][kWarp * XS];
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t c = tid / kChunkScan;
-  if (c >= lv.n_chunks) return;   // uniform per warp
-  const int j = (int)(tid - c * kChunkScan);
-  const int cnt = lv.count[c];
-  const bool active = j < cnt;
-  const int64_t i0 = lv.first[c];
-  const int64_t i = i0 + j;
-  const int flag = flag_in[c];
+  constexpr int REC = R::size, W = (R::g + NX + 3) / 4 * 4;
   const RowsPacked<T, NX> cin{(T*)carry_in};
-  T cg[NX], zD[NX * NX];
-#pragma unroll
-  for (int q = 0; q < NX * NX; ++q) zD[q] = T(0);
   if (!active) {
   } else if (j == cnt - 1) {
     cin.load_mean(c, cg);
@@ -168,29 +153,50 @@ smoother_down_cs_g(DevLevel lv, const T* __restrict__ items, const T* __restrict
   } else {
     load<T, NX>(items + (i + 1) * REC + R::g, cg);
   }
-  warp_store_carries<T, NX>(carry_out + i0 * XS, SO[threadIdx.x / kWarp], cg, zD, j, cnt,
-                            active);
-  if (active) flag_out[i] = j == cnt - 1 ? flag : 1;
+  return j == cnt - 1 ? flag != 0 : true;
 }
 
-// Leaf down-sweep (see smoother_leaf_down with add_nominal), means only: the
+// Chunk down-sweep (see smoother_down_cs), g only: each item's carry g.
+template <typename T, int NX>
+__global__ void __launch_bounds__(kBlock)
+smoother_down_cs_g(DevLevel lv, const T* __restrict__ items, const T* __restrict__ carry_in,
+                   const int* __restrict__ flag_in, T* __restrict__ carry_out,
+                   int* __restrict__ flag_out) {
+  constexpr int XS = XRow<NX>::size;
+  static_assert(kChunkScan == kWarp && kBlock % kWarp == 0, "one chunk per warp");
+  __shared__ __align__(16) T SO[kBlock / kWarp][kWarp * XS];
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t c = tid / kChunkScan;
+  if (c >= lv.n_chunks) return;   // uniform per warp
+  const int j = (int)(tid - c * kChunkScan);
+  const int cnt = lv.count[c];
+  const bool active = j < cnt;
+  const int64_t i0 = lv.first[c];
+  const int64_t i = i0 + j;
+  T cg[NX], zD[NX * NX];
+#pragma unroll
+  for (int q = 0; q < NX * NX; ++q) zD[q] = T(0);
+  const bool have =
+      smoother_item_carry_g<T, NX>(items, carry_in, flag_in[c], c, i, j, cnt, active, cg);
+  warp_store_carries<T, NX>(carry_out + i0 * XS, SO[threadIdx.x / kWarp], cg, zD, j, cnt,
+                            active);
+  if (active) flag_out[i] = have;
+}
+
+// Leaf steps (see smoother_leaf_steps with add_nominal), means only: the
 // RTS steps' g from the stored E_k, the new nominal mean (previous + the
 // deviation) written into the mean words of each row, its factor words kept.
 template <typename T, int NX, int NY, typename GV, typename FO>
-__global__ void __launch_bounds__(kBlock)
-smoother_leaf_down_g(DevLevel lv, DevSeqs sq, GV gv, FO fo, const T* __restrict__ etab,
-                     const T* __restrict__ carry, const int* __restrict__ flag,
-                     RowsPacked<T, NX> out_rows, int* status) {
-  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (c >= lv.n_chunks) return;
+SQSM_DEV void smoother_leaf_steps_g(const DevLevel& lv, const DevSeqs& sq, const GV& gv,
+                                    const FO& fo, const T* __restrict__ etab,
+                                    const RowsPacked<T, NX>& out_rows, int* status,
+                                    const PriorMean<T>& pm, int64_t c, T* gm) {
   constexpr int ES = ETab<NX>::size, MV = XRow<NX>::mvec, XS = XRow<NX>::size;
   const int b = lv.seq[c];
   const int64_t e0 = lv.first[c];
   const int cnt = lv.count[c];
   const int64_t r0 = sq.offsets[b] + b;
   const int64_t nb = sq.offsets[b + 1] - sq.offsets[b];
-  T gm[NX];
-  if (flag[c]) RowsPacked<T, NX>{(T*)carry}.load_mean(c, gm);
   bool ok = true;
   for (int j = cnt - 1; j >= 0; --j) {
     const int64_t e = e0 + j;
@@ -215,10 +221,46 @@ smoother_leaf_down_g(DevLevel lv, DevSeqs sq, GV gv, FO fo, const T* __restrict_
 #pragma unroll
     for (int i = 0; i < NX; ++i) w[i] = w[i] + gm[i];
     vstore<T, MV>(row, w);
+    if (k == 0 && pm.dm0) {
+#pragma unroll
+      for (int i = 0; i < NX; ++i) pm.dm0[(int64_t)b * NX + i] = pm.m0[(int64_t)b * NX + i] - w[i];
+    }
 #pragma unroll
     for (int i = 0; i < NX; ++i) ok = ok && finite(gm[i]);
   }
   if (!ok) flag_status(status, 8);
+}
+
+template <typename T, int NX, int NY, typename GV, typename FO>
+__global__ void __launch_bounds__(kBlock)
+smoother_leaf_down_g(DevLevel lv, DevSeqs sq, GV gv, FO fo, const T* __restrict__ etab,
+                     const T* __restrict__ carry, const int* __restrict__ flag,
+                     RowsPacked<T, NX> out_rows, int* status, PriorMean<T> pm) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= lv.n_chunks) return;
+  T gm[NX];
+  if (flag[c]) RowsPacked<T, NX>{(T*)carry}.load_mean(c, gm);
+  smoother_leaf_steps_g<T, NX, NY, GV, FO>(lv, sq, gv, fo, etab, out_rows, status, pm, c, gm);
+}
+
+// Level 1's chunk down-sweep and the leaf's in one launch (see
+// smoother_down_leaf), means only.
+template <typename T, int NX, int NY, typename GV, typename FO>
+__global__ void __launch_bounds__(kBlock)
+smoother_down_leaf_g(DevLevel lv, const T* __restrict__ items, const T* __restrict__ carry_in,
+                     const int* __restrict__ flag_in, DevLevel leaf, DevSeqs sq, GV gv, FO fo,
+                     const T* __restrict__ etab, RowsPacked<T, NX> out_rows, int* status,
+                     PriorMean<T> pm) {
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t c = tid / kChunkScan;
+  if (c >= lv.n_chunks) return;
+  const int j = (int)(tid - c * kChunkScan);
+  const int cnt = lv.count[c];
+  if (j >= cnt) return;
+  const int64_t i = lv.first[c] + j;
+  T gm[NX];
+  smoother_item_carry_g<T, NX>(items, carry_in, flag_in[c], c, i, j, cnt, true, gm);
+  smoother_leaf_steps_g<T, NX, NY, GV, FO>(leaf, sq, gv, fo, etab, out_rows, status, pm, i, gm);
 }
 
 // Enqueues the mean-only smoother scan when the sequences span more than one
@@ -229,7 +271,7 @@ smoother_leaf_down_g(DevLevel lv, DevSeqs sq, GV gv, FO fo, const T* __restrict_
 template <typename T, int NX, int NY, typename GV, typename FO>
 bool enqueue_smoother_means(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv, FO fo,
                             RowsPacked<T, NX> so, const T* etab, int* status, cudaStream_t s,
-                            Prof* P = nullptr) {
+                            Prof* P = nullptr, PriorMean<T> pm = {}) {
   const int Lc = (int)L.lv.size();
   constexpr int KS = KsMax<T, SRec<NX>::size>::value;
   const int Lk = L.ks_level(KS);
@@ -251,15 +293,21 @@ bool enqueue_smoother_means(const LevelSet& L, const ScanBuffers& W, DevSeqs sq,
     smoother_top_ks_g<T, NX><<<L.B, KS, 0, s>>>(L.seq_item_off[Lk], (const T*)W.items[Lk],
                                                 (T*)W.carry[Lk], W.flag[Lk]);
   }
-  for (int l = Lk - 1; l >= 1; --l) {
+  const bool fused = fuse_down(L, Lk);
+  for (int l = Lk - 1; l >= (fused ? 2 : 1); --l) {
     ProfScope ps(P, K_SMOOTHER_DOWN, s);
     smoother_down_cs_g<T, NX><<<cs_down_grid(L.lv[l].n_chunks), kBlock, 0, s>>>(
         L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1], W.flag[l + 1],
         (T*)W.carry[l], W.flag[l]);
   }
   ProfScope ps(P, K_SMOOTHER_LEAF_DOWN, s);
-  smoother_leaf_down_g<T, NX, NY, GV, FO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
-      L.lv[0], sq, gv, fo, etab, (const T*)W.carry[1], W.flag[1], so, status);
+  if (fused)
+    smoother_down_leaf_g<T, NX, NY, GV, FO><<<cs_down_grid(L.lv[1].n_chunks), kBlock, 0, s>>>(
+        L.lv[1], (const T*)W.items[1], (const T*)W.carry[2], W.flag[2], L.lv[0], sq, gv, fo, etab,
+        so, status, pm);
+  else
+    smoother_leaf_down_g<T, NX, NY, GV, FO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
+      L.lv[0], sq, gv, fo, etab, (const T*)W.carry[1], W.flag[1], so, status, pm);
   return true;
 }
 

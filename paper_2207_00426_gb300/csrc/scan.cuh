@@ -142,24 +142,20 @@ filter_down(DevLevel lv, const T* __restrict__ items, const T* __restrict__ carr
   }
 }
 
-// Leaf down-sweep: sequential square-root Kalman steps from the chunk's
-// carry (or from the prior (m0, N0) for the first chunk of a sequence),
-// writing m^f, N^f and the chunk's partial log-likelihood (FP64 sum).
+// Sequential square-root Kalman steps over leaf chunk c from its carry
+// (m, N) (have_carry), or from the prior (m0, N0) for the first chunk of a
+// sequence, writing m^f, N^f and the chunk's partial log-likelihood (FP64
+// sum).
 template <typename T, int NX, int NY, typename GV, typename FO>
-__global__ void __launch_bounds__(kBlock)
-filter_leaf_down(DevLevel lv, DevSeqs sq, GV gv, const T* __restrict__ y,
-                 const T* __restrict__ m0, const T* __restrict__ N0,
-                 const T* __restrict__ carry, const int* __restrict__ flag,
-                 FO fo, double* __restrict__ partial, int* status) {
-  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (c >= lv.n_chunks) return;
+SQSM_DEV void filter_leaf_steps(const DevLevel& lv, const DevSeqs& sq, const GV& gv,
+                                const T* __restrict__ y, const T* __restrict__ m0,
+                                const T* __restrict__ N0, const FO& fo,
+                                double* __restrict__ partial, int* status, int64_t c,
+                                bool have_carry, T* m, T* N) {
   const int b = lv.seq[c];
   const int64_t s0 = lv.first[c];
   const int cnt = lv.count[c];
-  T m[NX], N[NX * NX];
-  if (flag[c]) {
-    RowsPacked<T, NX>{(T*)carry}.load(c, m, N);
-  } else {
+  if (!have_carry) {
     load<T, NX>(m0 + (int64_t)b * NX, m);
     load_lower<T, NX>(N0 + (int64_t)b * NX * NX, N);
     fo.store(sq.offsets[b] + b, m, N);   // k = 0
@@ -180,6 +176,21 @@ filter_leaf_down(DevLevel lv, DevSeqs sq, GV gv, const T* __restrict__ y,
   }
   if (partial) partial[c] = acc;
   if (!ok) flag_status(status, 8);
+}
+
+// Leaf down-sweep: one thread per leaf chunk.
+template <typename T, int NX, int NY, typename GV, typename FO>
+__global__ void __launch_bounds__(kBlock)
+filter_leaf_down(DevLevel lv, DevSeqs sq, GV gv, const T* __restrict__ y,
+                 const T* __restrict__ m0, const T* __restrict__ N0,
+                 const T* __restrict__ carry, const int* __restrict__ flag,
+                 FO fo, double* __restrict__ partial, int* status) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= lv.n_chunks) return;
+  T m[NX], N[NX * NX];
+  const bool have = flag[c] != 0;
+  if (have) RowsPacked<T, NX>{(T*)carry}.load(c, m, N);
+  filter_leaf_steps<T, NX, NY, GV, FO>(lv, sq, gv, y, m0, N0, fo, partial, status, c, have, m, N);
 }
 
 // ---------------------------------------------------------------------------
@@ -278,20 +289,23 @@ smoother_down(DevLevel lv, const T* __restrict__ items, const T* __restrict__ ca
   }
 }
 
-// Leaf down-sweep: sequential square-root RTS steps from the chunk's carry
+// Sequential square-root RTS steps over leaf chunk c from its carry (gm, Dm)
 // (m^s, N^s just after the chunk), writing m^s, N^s to `out_rows`.  With
 // add_nominal the scan runs on deviations from a nominal trajectory held in
 // `out_rows` itself, and the written mean is nominal + deviation (each row is
 // read, then written, by the same thread); with dmax set, the largest
 // change of a mean from the one held in `out_rows` (the deviation, with
-// add_nominal) is max-reduced over all rows into *dmax (float bits).
+// add_nominal) is max-reduced over all rows into *dmax (float bits).  With
+// prior.dm0 set, the thread of a sequence's first row also writes the next
+// pass's prior mean in deviation coordinates (m0 minus the new mean).
+template <typename T> struct PriorMean {
+  const T* m0;
+  T* dm0;
+};
 template <typename T, int NX, int NY, typename GV, typename FO, typename SO>
-__global__ void __launch_bounds__(kBlock)
-smoother_leaf_down(DevLevel lv, DevSeqs sq, GV gv, FO fo, const T* __restrict__ carry,
-                   const int* __restrict__ flag, SO out_rows, int* status, bool add_nominal,
-                   unsigned* dmax) {
-  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (c >= lv.n_chunks) return;
+SQSM_DEV void smoother_leaf_steps(const DevLevel& lv, const DevSeqs& sq, const GV& gv,
+                                  const FO& fo, const SO& out_rows, int* status, bool add_nominal,
+                                  unsigned* dmax, const PriorMean<T>& prior, int64_t c, T* gm, T* Dm) {
   constexpr int REC = SRec<NX>::size;
   const int b = lv.seq[c];
   const int64_t e0 = lv.first[c];
@@ -299,8 +313,6 @@ smoother_leaf_down(DevLevel lv, DevSeqs sq, GV gv, FO fo, const T* __restrict__ 
   const int64_t r0 = sq.offsets[b] + b;
   const int64_t nb = sq.offsets[b + 1] - sq.offsets[b];
   float change = 0.f;
-  T gm[NX], Dm[NX * NX];
-  if (flag[c]) RowsPacked<T, NX>{(T*)carry}.load(c, gm, Dm);
   bool ok = true;
   // The inputs of a step (filter row, transition record, the mean held in
   // out_rows) do not depend on the steps after it, so each iteration issues
@@ -336,6 +348,11 @@ smoother_leaf_down(DevLevel lv, DevSeqs sq, GV gv, FO fo, const T* __restrict__ 
 #pragma unroll
       for (int i = 0; i < NX; ++i) out[i] = old[i] + gm[i];
       out_rows.store(e, out, Dm);
+      if (k == 0 && prior.dm0) {
+#pragma unroll
+        for (int i = 0; i < NX; ++i)
+          prior.dm0[(int64_t)b * NX + i] = prior.m0[(int64_t)b * NX + i] - out[i];
+      }
       if (dmax) {
 #pragma unroll
         for (int i = 0; i < NX; ++i) change = fmaxf(change, fabsf((float)gm[i]));
@@ -365,6 +382,20 @@ smoother_leaf_down(DevLevel lv, DevSeqs sq, GV gv, FO fo, const T* __restrict__ 
     bits = __reduce_max_sync(mask, bits);
     if ((int)(threadIdx.x & 31) == __ffs(mask) - 1) atomicMax(dmax, bits);
   }
+}
+
+// Leaf down-sweep: one thread per leaf chunk.
+template <typename T, int NX, int NY, typename GV, typename FO, typename SO>
+__global__ void __launch_bounds__(kBlock)
+smoother_leaf_down(DevLevel lv, DevSeqs sq, GV gv, FO fo, const T* __restrict__ carry,
+                   const int* __restrict__ flag, SO out_rows, int* status, bool add_nominal,
+                   unsigned* dmax, PriorMean<T> pm) {
+  const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (c >= lv.n_chunks) return;
+  T gm[NX], Dm[NX * NX];
+  if (flag[c]) RowsPacked<T, NX>{(T*)carry}.load(c, gm, Dm);
+  smoother_leaf_steps<T, NX, NY, GV, FO, SO>(lv, sq, gv, fo, out_rows, status, add_nominal, dmax,
+                                             pm, c, gm, Dm);
 }
 
 }  // namespace sqsm

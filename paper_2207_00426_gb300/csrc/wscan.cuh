@@ -336,25 +336,15 @@ SQSM_DEV void warp_store_rows(T* __restrict__ g, T* sh, const T* v, int j, int c
   for (int k = lane; k < cnt * W; k += kWarp) g[k] = sh[k];
 }
 
-// One thread per item of the level; each warp is one chunk.
+// The carry of item j of chunk c of a chunk-scanned level (one warp per
+// chunk, lane j): the chunk's carry applied to the in-chunk prefix before the
+// item, that prefix itself where the chunk starts its sequence (flag 0).
+// Returns whether the item has a carry.
 template <typename T, int NX>
-__global__ void __launch_bounds__(kBlock)
-filter_down_cs(DevLevel lv, const T* __restrict__ items, const T* __restrict__ carry_in,
-               const int* __restrict__ flag_in, T* __restrict__ carry_out, int* __restrict__ flag_out) {
-  constexpr int REC = FRec<NX>::size, XS = XRow<NX>::size;
-  static_assert(kChunkScan == kWarp && kBlock % kWarp == 0, "one chunk per warp");
-  __shared__ __align__(16) T SO[kBlock / kWarp][kWarp * XS];
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t c = tid / kChunkScan;
-  if (c >= lv.n_chunks) return;   // uniform per warp
-  const int j = (int)(tid - c * kChunkScan);
-  const int cnt = lv.count[c];
-  const bool active = j < cnt;
-  const int64_t i0 = lv.first[c];
-  const int64_t i = i0 + j;
-  const int flag = flag_in[c];
+SQSM_DEV bool filter_item_carry(const T* __restrict__ items, const T* __restrict__ carry_in,
+                                int flag, int64_t c, int64_t i, int j, bool active, T* cb, T* cU) {
+  constexpr int REC = FRec<NX>::size;
   const RowsPacked<T, NX> cin{(T*)carry_in};
-  T cb[NX], cU[NX * NX];
   if (!active) {
   } else if (j == 0) {
     cin.load(c, cb, cU);
@@ -367,9 +357,56 @@ filter_down_cs(DevLevel lv, const T* __restrict__ items, const T* __restrict__ c
     load<T, NX>(items + (i - 1) * REC + FRec<NX>::b, cb);
     load<T, NX * NX>(items + (i - 1) * REC + FRec<NX>::U, cU);
   }
+  return j == 0 ? flag != 0 : true;
+}
+
+// One thread per item of the level; each warp is one chunk.
+template <typename T, int NX>
+__global__ void __launch_bounds__(kBlock)
+filter_down_cs(DevLevel lv, const T* __restrict__ items, const T* __restrict__ carry_in,
+               const int* __restrict__ flag_in, T* __restrict__ carry_out, int* __restrict__ flag_out) {
+  constexpr int XS = XRow<NX>::size;
+  static_assert(kChunkScan == kWarp && kBlock % kWarp == 0, "one chunk per warp");
+  __shared__ __align__(16) T SO[kBlock / kWarp][kWarp * XS];
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t c = tid / kChunkScan;
+  if (c >= lv.n_chunks) return;   // uniform per warp
+  const int j = (int)(tid - c * kChunkScan);
+  const int cnt = lv.count[c];
+  const bool active = j < cnt;
+  const int64_t i0 = lv.first[c];
+  const int64_t i = i0 + j;
+  T cb[NX], cU[NX * NX];
+  const bool have = filter_item_carry<T, NX>(items, carry_in, flag_in[c], c, i, j, active, cb, cU);
   warp_store_carries<T, NX>(carry_out + i0 * XS, SO[threadIdx.x / kWarp], cb, cU, j, cnt,
                             active);
-  if (active) flag_out[i] = j == 0 ? flag : 1;
+  if (active) flag_out[i] = have;
+}
+
+// filter_down_cs of level 1 and filter_leaf_down in one launch: item i of the
+// level is leaf chunk i, so its thread goes on with the chunk's steps and the
+// carries stay in registers.  For scans of at most 65536 leaf chunks, where
+// the two launches and the carries' way through memory cost more than the
+// lower occupancy: with the smoother's pair a track of n = 1000 takes 98 ->
+// 90 us an iteration, of 1e5 (two passes) 336 -> 323, the population model at
+// n = 10000 27 -> 23.  A batch whose chunks leave lanes idle would spread its
+// leaf steps over more warps and keeps the two.
+template <typename T, int NX, int NY, typename GV, typename FO>
+__global__ void __launch_bounds__(kBlock)
+filter_down_leaf(DevLevel lv, const T* __restrict__ items, const T* __restrict__ carry_in,
+                 const int* __restrict__ flag_in, DevLevel leaf, DevSeqs sq, GV gv,
+                 const T* __restrict__ y, const T* __restrict__ m0, const T* __restrict__ N0,
+                 FO fo, double* __restrict__ partial, int* status) {
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t c = tid / kChunkScan;
+  if (c >= lv.n_chunks) return;
+  const int j = (int)(tid - c * kChunkScan);
+  if (j >= lv.count[c]) return;
+  const int64_t i = lv.first[c] + j;
+  T m[NX], N[NX * NX];
+  const bool have = filter_item_carry<T, NX>(items, carry_in, flag_in[c], c, i, j, true, m, N);
+  filter_leaf_steps<T, NX, NY, GV, FO>(leaf, sq, gv, y, m0, N0, fo, partial, status, i, have, m,
+                                       N);
 }
 
 template <typename T, int NX>
@@ -396,24 +433,13 @@ smoother_up_cs(DevLevel lv, T* __restrict__ items, T* __restrict__ out) {
   if (t == 0 && cnt > 0) vstore<T, REC>(out + c * REC, mine);
 }
 
+// As filter_item_carry, for the smoother's suffixes.
 template <typename T, int NX>
-__global__ void __launch_bounds__(kBlock)
-smoother_down_cs(DevLevel lv, const T* __restrict__ items, const T* __restrict__ carry_in,
-                 const int* __restrict__ flag_in, T* __restrict__ carry_out, int* __restrict__ flag_out) {
-  constexpr int REC = SRec<NX>::size, XS = XRow<NX>::size;
-  static_assert(kChunkScan == kWarp && kBlock % kWarp == 0, "one chunk per warp");
-  __shared__ __align__(16) T SO[kBlock / kWarp][kWarp * XS];
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t c = tid / kChunkScan;
-  if (c >= lv.n_chunks) return;   // uniform per warp
-  const int j = (int)(tid - c * kChunkScan);
-  const int cnt = lv.count[c];
-  const bool active = j < cnt;
-  const int64_t i0 = lv.first[c];
-  const int64_t i = i0 + j;
-  const int flag = flag_in[c];
+SQSM_DEV bool smoother_item_carry(const T* __restrict__ items, const T* __restrict__ carry_in,
+                                  int flag, int64_t c, int64_t i, int j, int cnt, bool active,
+                                  T* cg, T* cD) {
+  constexpr int REC = SRec<NX>::size;
   const RowsPacked<T, NX> cin{(T*)carry_in};
-  T cg[NX], cD[NX * NX];
   if (!active) {
   } else if (j == cnt - 1) {
     cin.load(c, cg, cD);
@@ -426,9 +452,50 @@ smoother_down_cs(DevLevel lv, const T* __restrict__ items, const T* __restrict__
     load<T, NX>(items + (i + 1) * REC + SRec<NX>::g, cg);
     load<T, NX * NX>(items + (i + 1) * REC + SRec<NX>::D, cD);
   }
+  return j == cnt - 1 ? flag != 0 : true;
+}
+
+template <typename T, int NX>
+__global__ void __launch_bounds__(kBlock)
+smoother_down_cs(DevLevel lv, const T* __restrict__ items, const T* __restrict__ carry_in,
+                 const int* __restrict__ flag_in, T* __restrict__ carry_out, int* __restrict__ flag_out) {
+  constexpr int XS = XRow<NX>::size;
+  static_assert(kChunkScan == kWarp && kBlock % kWarp == 0, "one chunk per warp");
+  __shared__ __align__(16) T SO[kBlock / kWarp][kWarp * XS];
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t c = tid / kChunkScan;
+  if (c >= lv.n_chunks) return;   // uniform per warp
+  const int j = (int)(tid - c * kChunkScan);
+  const int cnt = lv.count[c];
+  const bool active = j < cnt;
+  const int64_t i0 = lv.first[c];
+  const int64_t i = i0 + j;
+  T cg[NX], cD[NX * NX];
+  const bool have =
+      smoother_item_carry<T, NX>(items, carry_in, flag_in[c], c, i, j, cnt, active, cg, cD);
   warp_store_carries<T, NX>(carry_out + i0 * XS, SO[threadIdx.x / kWarp], cg, cD, j, cnt,
                             active);
-  if (active) flag_out[i] = j == cnt - 1 ? flag : 1;
+  if (active) flag_out[i] = have;
+}
+
+// smoother_down_cs of level 1 and smoother_leaf_down in one launch (see
+// filter_down_leaf).
+template <typename T, int NX, int NY, typename GV, typename FO, typename SO>
+__global__ void __launch_bounds__(kBlock)
+smoother_down_leaf(DevLevel lv, const T* __restrict__ items, const T* __restrict__ carry_in,
+                   const int* __restrict__ flag_in, DevLevel leaf, DevSeqs sq, GV gv, FO fo,
+                   SO out_rows, int* status, bool add_nominal, unsigned* dmax, PriorMean<T> pm) {
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t c = tid / kChunkScan;
+  if (c >= lv.n_chunks) return;
+  const int j = (int)(tid - c * kChunkScan);
+  const int cnt = lv.count[c];
+  if (j >= cnt) return;
+  const int64_t i = lv.first[c] + j;
+  T gm[NX], Dm[NX * NX];
+  smoother_item_carry<T, NX>(items, carry_in, flag_in[c], c, i, j, cnt, true, gm, Dm);
+  smoother_leaf_steps<T, NX, NY, GV, FO, SO>(leaf, sq, gv, fo, out_rows, status, add_nominal, dmax,
+                                             pm, i, gm, Dm);
 }
 
 inline unsigned cs_down_grid(int64_t chunks) {
