@@ -634,13 +634,24 @@ template <typename T, int LIN> constexpr int slr_min_blocks() {
   return sizeof(T) == 4 && LIN != 3 ? 5 : 1;
 }
 
+// In FP64 a step is two threads of different blocks, one for its transition
+// and one for its observation: a short track's time is the FP64 instructions of
+// one thread (n = 4000: 76 -> 53 us).  FP32 fills the GPU's schedulers with
+// one thread per step at the lengths that take long (1.04e7 steps: 1416 us,
+// split 1728).
+template <typename T> struct SlrSplit { static constexpr bool value = sizeof(T) == 8; };
+
 template <typename T, bool PACKED, typename NO, int LIN, bool TB = false>
 __global__ void __launch_bounds__(kBlock, (slr_min_blocks<T, LIN>()))
 ct_slr_kernel_lin(DevLevel lv, int leaf, DevSeqs sq, const CTParams<T>* __restrict__ Pp,
               int centered, NO nom, const T* __restrict__ y, T* __restrict__ F,
               T* __restrict__ c, T* __restrict__ SQo, T* __restrict__ H, T* __restrict__ d,
               T* __restrict__ SRo) {
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  // SPLIT: even blocks linearise the transitions of their steps, odd blocks
+  // the observations
+  constexpr bool SPLIT = SlrSplit<T>::value;
+  const bool obs = SPLIT && (blockIdx.x & 1);
+  const int64_t tid = (blockIdx.x >> (SPLIT ? 1 : 0)) * (int64_t)blockDim.x + threadIdx.x;
   const int64_t ch = tid / leaf;
   if (ch >= lv.n_chunks) return;
   const int j = (int)(tid - ch * leaf);
@@ -651,7 +662,7 @@ ct_slr_kernel_lin(DevLevel lv, int leaf, DevSeqs sq, const CTParams<T>* __restri
   const int64_t s = lv.first[ch] + j;
   const int64_t rp = s + b, rk = s + b + 1;
   T m[NX], N[NX * NX];
-  {   // transition at k - 1
+  if (!SPLIT || !obs) {   // transition at k - 1
     nom.load(rp, m, N);
     T Fm[NX * NX], cm[NX], Sl[NX * NX];
     T fm[NX];    // f(m_{k-1}) (absolute) or f(m_{k-1}) - m_k (deviation form)
@@ -702,7 +713,7 @@ ct_slr_kernel_lin(DevLevel lv, int leaf, DevSeqs sq, const CTParams<T>* __restri
       store_lower<T, NX>(SQo + s * NX * NX, Sl);
     }
   }
-  {   // observation at k
+  if (!SPLIT || obs) {   // observation at k
     nom.load(rk, m, N);
     T hm[NY], Hm[NY * NX], dm[NY], So[NY * NY], ys[NY];
     load<T, NY>(y + s * NY, ys);
@@ -991,32 +1002,32 @@ void launch_ct_slr(unsigned grid, cudaStream_t s, int linearization, DevLevel lv
                    DevSeqs sq, const CTParams<T>* Pp, int centered, NO nom, const T* y, T* F,
                    T* c, T* SQo, T* H, T* d, T* SRo, int textbook = 0) {
   if (textbook && linearization == 0) {
-    ct_slr_kernel_lin<T, PACKED, NO, 0, true><<<grid, kBlock, 0, s>>>(lv, leaf, sq, Pp, centered,
+    ct_slr_kernel_lin<T, PACKED, NO, 0, true><<<(SlrSplit<T>::value ? 2 : 1) * grid, kBlock, 0, s>>>(lv, leaf, sq, Pp, centered,
                                                                        nom, y, F, c, SQo, H, d,
                                                                        SRo);
     return;
   }
   switch (linearization) {
     case 0:
-      ct_slr_kernel_lin<T, PACKED, NO, 0><<<grid, kBlock, 0, s>>>(lv, leaf, sq, Pp, centered, nom,
+      ct_slr_kernel_lin<T, PACKED, NO, 0><<<(SlrSplit<T>::value ? 2 : 1) * grid, kBlock, 0, s>>>(lv, leaf, sq, Pp, centered, nom,
                                                                    y, F, c, SQo, H, d, SRo);
       break;
     case 2:
-      ct_slr_kernel_lin<T, PACKED, NO, 2><<<grid, kBlock, 0, s>>>(lv, leaf, sq, Pp, centered, nom,
+      ct_slr_kernel_lin<T, PACKED, NO, 2><<<(SlrSplit<T>::value ? 2 : 1) * grid, kBlock, 0, s>>>(lv, leaf, sq, Pp, centered, nom,
                                                                    y, F, c, SQo, H, d, SRo);
       break;
     case 3:
-      // FP64 keeps one thread per step (the points' values would not
+      // FP64 keeps one thread per part of a step (the points' values would not
       // fit its registers)
       if constexpr (sizeof(T) == 4)
         ct_slr_gh_kernel<T, PACKED, NO><<<grid * kGhLanes, kBlock, 0, s>>>(
             lv, leaf, sq, Pp, centered, nom, y, F, c, SQo, H, d, SRo);
       else
-        ct_slr_kernel_lin<T, PACKED, NO, 3><<<grid, kBlock, 0, s>>>(
+        ct_slr_kernel_lin<T, PACKED, NO, 3><<<(SlrSplit<T>::value ? 2 : 1) * grid, kBlock, 0, s>>>(
             lv, leaf, sq, Pp, centered, nom, y, F, c, SQo, H, d, SRo);
       break;
     default:
-      ct_slr_kernel_lin<T, PACKED, NO, 1><<<grid, kBlock, 0, s>>>(lv, leaf, sq, Pp, centered, nom,
+      ct_slr_kernel_lin<T, PACKED, NO, 1><<<(SlrSplit<T>::value ? 2 : 1) * grid, kBlock, 0, s>>>(lv, leaf, sq, Pp, centered, nom,
                                                                    y, F, c, SQo, H, d, SRo);
       break;
   }
