@@ -530,6 +530,7 @@ SQSM_DEV void adj_slr_row(int64_t e, int b, const DevSeqs& sq, const CTParams<T>
   using GR = GRec<NX, NY>;
   using ST = SlrTab<NX, NY>;
   const CTParams<T> P = *Pp;
+  const CTGradParams& gp = *reinterpret_cast<const CTGradParams*>(Pp + 1);
   const int64_t k = e - (sq.offsets[b] + b);
   const int64_t nb = sq.offsets[b + 1] - sq.offsets[b];
   T m[NX], N[NX * NX], mb[NX], Nb[NX * NX];
@@ -563,12 +564,10 @@ SQSM_DEV void adj_slr_row(int64_t e, int b, const DevSeqs& sq, const CTParams<T>
     }
     // Q = q_c Q_c + q_w Q_w (Q_w only at (4, 4)): d/d log q_c = Lambda-bar :
     // (Q - Q_44 e_4 e_4^T), d/d log q_w = Lambda-bar_44 Q_44
-    T Q[NX * NX];
-    gram_lower<T, NX>(P.SQ, Q);
     double tq = 0.0;
 #pragma unroll
-    for (int i = 0; i < NX * NX; ++i) tq += (double)Lb[i] * (double)Q[i];
-    const double t44 = (double)Lb[24] * (double)Q[24];
+    for (int i = 0; i < 9; ++i) tq += (double)Lb[ct_q_at(i)] * gp.Q[i];
+    const double t44 = (double)Lb[24] * gp.Q[8];
     th[1] += tq - t44;
     th[2] += t44;
   }
@@ -595,8 +594,8 @@ SQSM_DEV void adj_slr_row(int64_t e, int b, const DevSeqs& sq, const CTParams<T>
           gb + GR::H, gb + GR::d, Lb, mb, Nb);
     }
     // Omega = diag(sigma_1^2, sigma_2^2): d/d log sigma_i = 2 sigma_i^2 Omega-bar_ii
-    th[0] += 2.0 * (double)P.sigma[0] * (double)P.sigma[0] * (double)Lb[0];
-    th[3] += 2.0 * (double)P.sigma[1] * (double)P.sigma[1] * (double)Lb[3];
+    th[0] += gp.two_var[0] * (double)Lb[0];
+    th[3] += gp.two_var[1] * (double)Lb[3];
   }
 #pragma unroll
   for (int i = 0; i < NX; ++i) o[i] = mb[i];
@@ -611,26 +610,31 @@ SQSM_DEV void adj_slr_row(int64_t e, int b, const DevSeqs& sq, const CTParams<T>
 }
 
 // Sum of four values over the block (kBlock threads) in a fixed order,
-// written by thread 0 to out[0..3].
-SQSM_DEV void block_sum4(double* v, double* __restrict__ out) {
+// written by thread 0 to out[0..3].  An FP64 addition holds an SM's unit for 19
+// cycles a warp, so the warp's sums are folded together: halves, then
+// quarters of the warp keep one value each (2 + 1 + 3 additions for 20).
+SQSM_DEV void block_sum4(const double* v, double* __restrict__ out) {
   __shared__ double part[kBlock / 32][4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_down_sync(0xffffffffu, v[j], o);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0)
+  const bool hi = lane & 16, hj = lane & 8;
+  double a[2];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) part[w][j] = v[j];
+  for (int j = 0; j < 2; ++j) {
+    const double keep = hi ? v[2 + j] : v[j], give = hi ? v[j] : v[2 + j];
+    a[j] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+  }
+  const double keep = hj ? a[1] : a[0], give = hj ? a[0] : a[1];
+  double s = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((lane & 7) == 0) part[w][lane >> 3] = s;   // value 2 hi + hj
   __syncthreads();
-  if (threadIdx.x == 0)
+  if (threadIdx.x < 4) {
+    double t = 0.0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      double t = 0.0;
-#pragma unroll
-      for (int q = 0; q < kBlock / 32; ++q) t += part[q][j];
-      out[j] = t;
-    }
+    for (int q = 0; q < kBlock / 32; ++q) t += part[q][threadIdx.x];
+    out[threadIdx.x] = t;
+  }
 }
 
 // One thread per state row (smoother leaf chunks of `leaf` rows); every

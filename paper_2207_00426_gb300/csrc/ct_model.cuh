@@ -39,6 +39,19 @@ struct CTParams {
   T SQ[25];      // lower Cholesky factor of the process noise
 };
 
+// What the gradient's FP64 parameter sums take from them (values rounded to T
+// first), behind the CTParams of a workspace.
+struct CTGradParams {
+  double Q[9];         // nonzeros of SQ SQ^T in row-major order (ct_q_at)
+  double two_var[2];   // 2 sigma^2 of each sensor
+};
+
+// Row-major positions of the nonzeros of the CT model's Q.
+__host__ __device__ constexpr int ct_q_at(int k) {
+  constexpr int at[9] = {0, 2, 6, 8, 10, 12, 16, 18, 24};
+  return at[k];
+}
+
 SQSM_DEV void sq_sincos(float a, float* s, float* c) { sincosf(a, s, c); }
 SQSM_DEV void sq_sincos(double a, double* s, double* c) { sincos(a, s, c); }
 SQSM_DEV float sq_atan2(float y, float x) { return atan2f(y, x); }
@@ -69,6 +82,16 @@ __global__ void ct_params_kernel(double th0, double th1, double th2, double th3,
     p.SQ[(i + 2) * 5 + i + 2] = (T)c;
   }
   p.SQ[24] = (T)sqrt(qw * dt);
+  CTGradParams g;
+  for (int k = 0; k < 9; ++k) {
+    const int i = ct_q_at(k) / 5, j = ct_q_at(k) % 5;
+    T s = T(0);
+    for (int q = 0; q <= (i < j ? i : j); ++q) s += p.SQ[i * 5 + q] * p.SQ[j * 5 + q];
+    g.Q[k] = (double)s;
+  }
+  for (int i = 0; i < 2; ++i) g.two_var[i] = 2.0 * (double)p.sigma[i] * (double)p.sigma[i];
+  static_assert(sizeof(CTParams<T>) % alignof(CTGradParams) == 0, "laid out one after the other");
+  *reinterpret_cast<CTGradParams*>(P + 1) = g;
   *P = p;
 }
 

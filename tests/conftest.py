@@ -1,3 +1,4 @@
+import gc
 import os
 import sys
 
@@ -11,3 +12,11 @@ if ROOT not in sys.path:
 def pytest_configure(config):
     config.addinivalue_line("markers", "gpu: needs a CUDA GPU (GB300, sm_103a)")
     config.addinivalue_line("markers", "slow: oracle runs that take tens of seconds")
+
+
+@pytest.fixture(autouse=True, scope="module")
+def _collect_contexts():
+    """A module's contexts give their device memory back before the next one
+    starts (a test there may compare the free memory before and after)."""
+    yield
+    gc.collect()
