@@ -174,6 +174,7 @@ bool build_levels(Plan& p, const std::vector<int64_t>& counts0, LevelSet& L, int
   std::vector<int64_t> counts = counts0;
   L.B = (int)counts0.size();
   L.lanes = p.lanes;
+  L.leaf = p.L0;
   int level = 0;
   int64_t total = 0;
   for (int64_t v : counts) total += v;

@@ -29,6 +29,7 @@ template <typename T, int NX> constexpr bool lane_forms() {
 // n_items[l] is the number of items at level l (n_items[Lc] = B).
 struct LevelSet {
   bool lanes = false;                  // upper levels in the lane forms
+  int leaf = 0;                        // steps per leaf chunk (0: not a context's plan)
   std::vector<DevLevel> lv;
   std::vector<int64_t> n_items;
   int64_t* leaf_chunk_off = nullptr;   // device, B+1
@@ -181,6 +182,19 @@ inline bool fuse_down(const LevelSet& L, int Lk) {
          4 * kChunkScan * L.lv[1].n_chunks <= 5 * L.n_items[1] + 4 * kChunkScan;
 }
 
+// Leaf kernels with a chunk's steps side by side (filter_leaf_up_par and the
+// smoother's): FP32 plans of kLeafPar steps per leaf and at most this many
+// leaf chunks.  Beyond, the chip is busy with one thread per chunk and the
+// blocks' barriers and idle warps cost more: four iterations over one track
+// of n = 49000 (16334 chunks) 574 -> 544 us, n = 70000 643 -> 652, n = 100000
+// 709 -> 756.
+constexpr int64_t kLeafParMaxChunks = 16384;
+
+template <typename T, int NX> bool leaf_par(const LevelSet& L) {
+  return sizeof(T) == 4 && NX >= kLaneMinNx && L.leaf == kLeafPar &&
+         L.lv[0].n_chunks <= kLeafParMaxChunks;
+}
+
 // Allow a kernel the dynamic shared memory of its next launch where that
 // exceeds the 48 KB default (a function attribute, not a stream operation,
 // so it may be set while the stream is being captured).
@@ -223,8 +237,17 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
   if (Lc > 1) {  // with one leaf chunk per sequence every carry is the prior
     {
       ProfScope ps(P, K_FILTER_LEAF_UP, s);
-      filter_leaf_up<T, NX, NY, GV><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
-          L.lv[0], sq, gv, y, m0, N0, (T*)W.items[1]);
+      bool par = false;
+      if constexpr (sizeof(T) == 4 && NX >= kLaneMinNx) {
+        par = leaf_par<T, NX>(L);
+        if (par)
+          filter_leaf_up_par<T, NX, NY, GV>
+              <<<(unsigned)((L.lv[0].n_chunks + kWarp - 1) / kWarp), kWarp * kLeafPar, 0, s>>>(
+                  L.lv[0], sq, gv, y, m0, N0, (T*)W.items[1]);
+      }
+      if (!par)
+        filter_leaf_up<T, NX, NY, GV><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
+            L.lv[0], sq, gv, y, m0, N0, (T*)W.items[1]);
     }
     for (int l = 1; l < Lk; ++l) {
       ProfScope ps(P, K_FILTER_UP, s);
@@ -348,8 +371,17 @@ void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv
   if (Lc > 1) {
     {
       ProfScope ps(P, K_SMOOTHER_LEAF_UP, s);
-      smoother_leaf_up<T, NX, NY, GV, FO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
-          L.lv[0], sq, gv, fo, (T*)W.items[1], etab);
+      bool par = false;
+      if constexpr (sizeof(T) == 4 && NX >= kLaneMinNx) {
+        par = leaf_par<T, NX>(L);
+        if (par)
+          smoother_leaf_up_par<T, NX, NY, GV, FO>
+              <<<(unsigned)((L.lv[0].n_chunks + kWarp - 1) / kWarp), kWarp * kLeafPar, 0, s>>>(
+                  L.lv[0], sq, gv, fo, (T*)W.items[1], etab);
+      }
+      if (!par)
+        smoother_leaf_up<T, NX, NY, GV, FO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
+            L.lv[0], sq, gv, fo, (T*)W.items[1], etab);
     }
     for (int l = 1; l < Lk; ++l) {
       ProfScope ps(P, K_SMOOTHER_UP, s);
@@ -422,6 +454,21 @@ void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv
           (T*)W.carry[l], W.flag[l]);
   }
   ProfScope ps(P, K_SMOOTHER_LEAF_DOWN, s);
+  if constexpr (sizeof(T) == 4 && NX >= kLaneMinNx) {
+    if (leaf_par<T, NX>(L)) {
+      constexpr int TH = kWarp * (kLeafPar + 1);
+      if (fused)
+        smoother_leaf_down_par<T, NX, NY, true, GV, FO, SO><<<(unsigned)L.lv[1].n_chunks, TH, 0, s>>>(
+            L.lv[1], (const T*)W.items[1], (const T*)W.carry[2], W.flag[2], L.lv[0], sq, gv, fo, so,
+            status, add_nominal, dmax, pm);
+      else
+        smoother_leaf_down_par<T, NX, NY, false, GV, FO, SO>
+            <<<(unsigned)((L.lv[0].n_chunks + kWarp - 1) / kWarp), TH, 0, s>>>(
+                L.lv[0], (const T*)nullptr, (const T*)W.carry[1], W.flag[1], L.lv[0], sq, gv, fo, so,
+                status, add_nominal, dmax, pm);
+      return;
+    }
+  }
   if (fused)
     smoother_down_leaf<T, NX, NY, GV, FO, SO><<<cs_down_grid(L.lv[1].n_chunks), kBlock, 0, s>>>(
         L.lv[1], (const T*)W.items[1], (const T*)W.carry[2], W.flag[2], L.lv[0], sq, gv, fo, so,

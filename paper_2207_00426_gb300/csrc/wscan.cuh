@@ -498,6 +498,222 @@ smoother_down_leaf(DevLevel lv, const T* __restrict__ items, const T* __restrict
                                              pm, i, gm, Dm);
 }
 
+// Leaf kernels of short FP32 scans with the steps of a leaf chunk side by
+// side: the elements of a chunk's kLeafPar rows do not depend on one another,
+// so each is built by a thread of its own warp (lane: chunk) and only the
+// combines, or the RTS steps, are one after another.  A call of a few thousand
+// steps has fewer warps than schedulers either way, and its leaf kernels take
+// one element's chain instead of three.  Same operations on the same values
+// as the one-thread kernels.  Four iterations over one track (us, one thread
+// against side by side): n = 300 344 -> 276, 3000 407 -> 329, 12000 490 -> 422,
+// 49000 574 -> 544; smoother of a linear model, n = 3000, 99 -> 79.
+constexpr int kLeafPar = 3;
+
+template <typename T, int NX, int NY, typename GV, typename FO>
+SQSM_DEV void smoother_row_element(const DevSeqs& sq, const GV& gv, const FO& fo, int b, int64_t e,
+                                   T* el) {
+  T m[NX], N[NX * NX];
+  const int64_t k = e - (sq.offsets[b] + b);
+  const int64_t nb = sq.offsets[b + 1] - sq.offsets[b];
+  fo.load(e, m, N);
+  if (k == nb) {
+    smoother_element_last<T, NX>(m, N, el);
+  } else {
+    Gamma<T, NX, NY> g;
+    g.load_transition(gv, sq.offsets[b] + k);
+    smoother_element<T, NX, NY>(g, m, N, el);
+  }
+}
+
+// See smoother_leaf_up.
+template <typename T, int NX, int NY, typename GV, typename FO>
+__global__ void __launch_bounds__(kWarp * kLeafPar)
+smoother_leaf_up_par(DevLevel lv, DevSeqs sq, GV gv, FO fo, T* __restrict__ items,
+                     T* __restrict__ etab) {
+  constexpr int REC = SRec<NX>::size;
+  __shared__ __align__(16) T S[kLeafPar][kWarp * REC];
+  const int lane = threadIdx.x % kWarp, j = threadIdx.x / kWarp;
+  const int64_t c = blockIdx.x * (int64_t)kWarp + lane;
+  const bool in = c < lv.n_chunks;
+  const int cnt = in ? lv.count[c] : 0;
+  if (j < cnt) {
+    const int b = lv.seq[c];
+    const int64_t e = lv.first[c] + j;
+    T el[REC];
+    smoother_row_element<T, NX, NY, GV, FO>(sq, gv, fo, b, e, el);
+    if (etab && e != sq.offsets[b + 1] + b)
+      vstore<T, ETab<NX>::size>(etab + e * ETab<NX>::size, el + SRec<NX>::E);
+    vstore<T, REC>(S[j] + lane * REC, el);
+  }
+  __syncthreads();
+  if (j == 0 && in) {
+    T agg[REC], el[REC], tmp[REC];
+    vload<T, REC>(S[cnt - 1] + lane * REC, agg);
+    for (int i = cnt - 2; i >= 0; --i) {
+      vload<T, REC>(S[i] + lane * REC, el);
+      smoother_combine<T, NX>(el, agg, tmp);
+      copy<T, REC>(tmp, agg);
+    }
+    vstore<T, REC>(items + c * REC, agg);
+  }
+}
+
+// See smoother_leaf_down and smoother_down_leaf (FUSED: lv is level 1 and a
+// block one of its chunks; otherwise carry / flag are the leaf chunks').  The
+// last warp takes the carry while the others build the elements.
+template <typename T, int NX, int NY, bool FUSED, typename GV, typename FO, typename SO>
+__global__ void __launch_bounds__(kWarp * (kLeafPar + 1))
+smoother_leaf_down_par(DevLevel lv, const T* __restrict__ items, const T* __restrict__ carry,
+                       const int* __restrict__ flag, DevLevel leaf, DevSeqs sq, GV gv, FO fo,
+                       SO out_rows, int* status, bool add_nominal, unsigned* dmax,
+                       PriorMean<T> prior) {
+  static_assert(kChunkScan == kWarp, "one chunk per block");
+  constexpr int REC = SRec<NX>::size;
+  __shared__ __align__(16) T S[kLeafPar][kWarp * REC];
+  const int lane = threadIdx.x % kWarp, w = threadIdx.x / kWarp;
+  int64_t c;
+  bool in;
+  if constexpr (FUSED) {
+    in = lane < lv.count[blockIdx.x];
+    c = lv.first[blockIdx.x] + lane;
+  } else {
+    c = blockIdx.x * (int64_t)kWarp + lane;
+    in = c < leaf.n_chunks;
+  }
+  const int cnt = in ? leaf.count[c] : 0;
+  const int b = in ? leaf.seq[c] : 0;
+  const int64_t e0 = in ? leaf.first[c] : 0;
+  const int64_t r0 = sq.offsets[b] + b, nb = sq.offsets[b + 1] - sq.offsets[b];
+  T gm[NX], Dm[NX * NX];
+  if (w < kLeafPar) {
+    if (w < cnt) {
+      T el[REC];
+      smoother_row_element<T, NX, NY, GV, FO>(sq, gv, fo, b, e0 + w, el);
+      vstore<T, REC>(S[w] + lane * REC, el);
+    }
+  } else if (in) {
+    if constexpr (FUSED)
+      smoother_item_carry<T, NX>(items, carry, flag[blockIdx.x], blockIdx.x, c, lane,
+                                 lv.count[blockIdx.x], true, gm, Dm);
+    else if (flag[c]) RowsPacked<T, NX>{(T*)carry}.load(c, gm, Dm);
+  }
+  __syncthreads();
+  if (w < kLeafPar || !in) return;
+  float change = 0.f;
+  bool ok = true;
+  const bool need_old = add_nominal || dmax != nullptr;
+  for (int j = cnt - 1; j >= 0; --j) {
+    const int64_t e = e0 + j;
+    T el[REC], old[NX], out[NX];
+    vload<T, REC>(S[j] + lane * REC, el);
+    if (need_old) out_rows.load_mean(e, old);
+    if (e - r0 == nb) {
+#pragma unroll
+      for (int i = 0; i < NX; ++i) gm[i] = el[SRec<NX>::g + i];
+#pragma unroll
+      for (int i = 0; i < NX * NX; ++i) Dm[i] = el[SRec<NX>::D + i];
+    } else {
+      smoother_apply<T, NX>(el, gm, Dm);
+    }
+#pragma unroll
+    for (int i = 0; i < NX; ++i) {
+      out[i] = add_nominal ? old[i] + gm[i] : gm[i];
+      if (dmax) change = fmaxf(change, fabsf((float)(add_nominal ? gm[i] : gm[i] - old[i])));
+      ok = ok && finite(gm[i]);
+    }
+    out_rows.store(e, out, Dm);
+    if (e == r0 && prior.dm0) {
+#pragma unroll
+      for (int i = 0; i < NX; ++i)
+        prior.dm0[(int64_t)b * NX + i] = prior.m0[(int64_t)b * NX + i] - out[i];
+    }
+  }
+  if (!ok) flag_status(status, 8);
+  if (dmax) {   // see smoother_leaf_steps
+    unsigned bits = __float_as_uint(ok ? change : INFINITY);
+    const unsigned mask = __activemask();
+    bits = __reduce_max_sync(mask, bits);
+    if (lane == __ffs(mask) - 1) atomicMax(dmax, bits);
+  }
+}
+
+// See filter_leaf_up: the elements side by side, then each combine by three
+// threads, one per part (see filter_ks3).
+template <typename T, int NX, int NY, typename GV>
+__global__ void __launch_bounds__(kWarp * kLeafPar)
+filter_leaf_up_par(DevLevel lv, DevSeqs sq, GV gv, const T* __restrict__ y,
+                   const T* __restrict__ m0, const T* __restrict__ N0, T* __restrict__ items) {
+  using R = FRec<NX>;
+  constexpr int REC = R::size, NZ = NX < NY ? NX : NY;
+  __shared__ __align__(16) T S[kLeafPar][kWarp * REC];
+  const int lane = threadIdx.x % kWarp, w = threadIdx.x / kWarp;
+  const int64_t c = blockIdx.x * (int64_t)kWarp + lane;
+  const bool in = c < lv.n_chunks;
+  const int cnt = in ? lv.count[c] : 0;
+  if (w < cnt) {
+    const int b = lv.seq[c];
+    const int64_t s = lv.first[c] + w;
+    T el[REC], ys[NY], m0b[NX], N0b[NX * NX];
+    load<T, NX>(m0 + (int64_t)b * NX, m0b);
+    load_lower<T, NX>(N0 + (int64_t)b * NX * NX, N0b);
+    Gamma<T, NX, NY> g;
+    g.load_all(gv, s);
+    load<T, NY>(y + s * NY, ys);
+    filter_element<T, NX, NY>(g, ys, s == sq.offsets[b], m0b, N0b, el);
+    if (cnt == 1) lower_Z<T, NX, NY>(el + R::Z);
+    vstore<T, REC>(S[w] + lane * REC, el);
+  }
+  __syncthreads();
+  T* agg = S[0] + lane * REC;
+  if constexpr (NX < 5) {
+    // (at n_x = 4 the parts' separate code would fuse other products than the
+    // whole combine's, and round differently)
+    if (w == 0 && cnt > 1) {
+      T acc[REC], el[REC], tmp[REC];
+      vload<T, REC>(agg, acc);
+      for (int i = 1; i < cnt; ++i) {
+        vload<T, REC>(S[i] + lane * REC, el);
+        filter_combine<T, NX, 7, true, NZ>(acc, el, tmp);
+        copy<T, REC>(tmp, acc);
+      }
+      vstore<T, REC>(agg, acc);
+    }
+    __syncthreads();
+  } else {
+    for (int i = 1; i < kLeafPar; ++i) {
+      T part[REC];
+      const T* ej = S[i] + lane * REC;
+      if (i < cnt) {
+        if (w == 0) filter_combine<T, NX, 1, true, NZ>(agg, ej, part);
+        else if (w == 1) filter_combine<T, NX, 2, true, NZ>(agg, ej, part);
+        else filter_combine<T, NX, 4, true, NZ>(agg, ej, part);
+      }
+      __syncthreads();
+      if (i < cnt) {
+        if (w == 0) {
+#pragma unroll
+          for (int k = R::A; k < R::U; ++k) agg[k] = part[k];
+#pragma unroll
+          for (int k = R::eta; k < R::Z; ++k) agg[k] = part[k];
+        } else if (w == 1) {
+#pragma unroll
+          for (int k = R::U; k < R::eta; ++k) agg[k] = part[k];
+        } else {
+#pragma unroll
+          for (int k = R::Z; k < R::Z + NX * NX; ++k) agg[k] = part[k];
+        }
+      }
+      __syncthreads();
+    }
+  }
+  // the block's chunks are consecutive: their records go out as one block
+  const int64_t c0 = blockIdx.x * (int64_t)kWarp;
+  const int n = lv.n_chunks - c0 < kWarp ? (int)(lv.n_chunks - c0) : kWarp;
+  const float4* S4 = reinterpret_cast<const float4*>(S[0]);
+  float4* I4 = reinterpret_cast<float4*>(items + c0 * REC);
+  for (int k = threadIdx.x; k < n * REC * (int)sizeof(T) / 16; k += blockDim.x) I4[k] = S4[k];
+}
+
 inline unsigned cs_down_grid(int64_t chunks) {
   return (unsigned)((chunks * kChunkScan + kBlock - 1) / kBlock);
 }
