@@ -99,6 +99,8 @@ void adj_enqueue(const IplsArgs& a, const AdjArgs& g, const LevelSet& Lf, const 
   // at most kAdjPerStepMaxLeaf - 1 maps), one per chunk for long ones
   const bool per_step = a.leaf <= kAdjPerStepMaxLeaf;
   const unsigned down_grid = grid_for(Lf.lv[0].n_chunks * (per_step ? a.leaf : 1));
+  const size_t down_smem = adj_leaf_down_smem<T>(per_step);
+  dyn_smem(adj_smoother_leaf_down<T>, down_smem);
   for (int it = 0; it < g.iters; ++it) {
     // smoother adjoint: forward-in-time scan of maps
     if (Lc > 1) {
@@ -109,7 +111,7 @@ void adj_enqueue(const IplsArgs& a, const AdjArgs& g, const LevelSet& Lf, const 
       cudaMemsetAsync(Wa.flag[Lc], 0, sizeof(int) * Lf.n_items[Lc], s);
     }
     adj_scan_down<T, true>(Lf, Wa, Lc > 1 ? Lk : Lc, s);
-    adj_smoother_leaf_down<T><<<down_grid, kBlock, 0, s>>>(
+    adj_smoother_leaf_down<T><<<down_grid, kBlock, down_smem, s>>>(
         Lf.lv[0], a.leaf, per_step, sq, ab, (const T*)Wa.carry[1], Wa.flag[1]);
     // filter adjoint: backward-in-time scan of maps
     if (Lc > 1) {

@@ -29,6 +29,27 @@ SQSM_DEV GammaPacked<T> gview(const AdjBufs& a) {
   return GammaPacked<T>{(T*)a.gam};
 }
 
+// Records of consecutive steps or rows, copied into a warp's shared memory by
+// its lanes in words of W floats (cp.async; one hardware wait, no spin).  A
+// lane's own record in global memory costs its warp one L1 line look-up per
+// lane and load (a 71-value record 2272 of them for 32 steps, 71 this way).
+template <int W> SQSM_DEV void warp_fetch(float* sh, const float* __restrict__ g, int n) {
+  const unsigned base = (unsigned)__cvta_generic_to_shared(sh);
+  for (int k = (threadIdx.x % kWarp) * W; k < n; k += kWarp * W) {
+    if constexpr (W == 4)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(base + 4u * k), "l"(g + k)
+                   : "memory");
+    else
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(base + 4u * k), "l"(g + k)
+                   : "memory");
+  }
+}
+
+SQSM_DEV void warp_fetch_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncwarp();
+}
+
 // --------------------------- per-step tables --------------------------------
 
 // One thread per time step (leaf chunks of `leaf` steps): the KfTab, RtsTab
@@ -135,9 +156,14 @@ adj_smoother_leaf_down(DevLevel lv, int leaf, bool per_step, DevSeqs sq, AdjBufs
   constexpr int NX = 5, NY = 2, X = XRec<NX>::size, REC = MapRec<NX>::size;
   using GR = GRec<NX, NY>;
   using RT = RtsTab<NX>;
-  // FP32 writes the gbar records of a warp's steps through shared memory
+  // FP32 reads the table records of a warp's steps and writes their gbar
+  // records and dfilt rows through shared memory (adj_leaf_down_smem): with a
+  // lane per record the L1's line look-ups bound the kernel (75% of its
+  // cycles); 512000 steps 226 -> 174 us.
   constexpr bool STAGE = sizeof(T) == 4;
-  __shared__ T SG[STAGE ? kBlock * GR::size : 1];
+  extern __shared__ __align__(16) unsigned char adj_smem[];
+  const int lane = threadIdx.x % kWarp;
+  T* const sh = (T*)adj_smem + (threadIdx.x / kWarp) * kWarp * (RT::size + GR::size);
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t c = per_step ? tid / leaf : tid;
   const bool in = c < lv.n_chunks;
@@ -152,24 +178,22 @@ adj_smoother_leaf_down(DevLevel lv, int leaf, bool per_step, DevSeqs sq, AdjBufs
     if (flag[c]) load<T, X>(carry + c * X, x);
     else load<T, X>((const T*)a.dir + (s0 + b) * X, x);
   }
-  // The RTS VJP of step j (the expensive part), writing its record part
-  // F | c | Lambda at go, and the map that carries the cotangent from step j
-  // to j + 1.
-  auto vjp = [&](int j, T* go) {
+  // The RTS VJP of step j (the expensive part) from its table record rtg: the
+  // record part F | c | Lambda at go and the row's direct cotangents df; and
+  // the map that carries the cotangent from step j to j + 1.
+  auto vjp = [&](int j, const T* rtg, T* go, T* df) {
     const int64_t s = s0 + j, e = s + b;
-    const T* rtg = (const T*)a.rtab + s * RT::size;
     Gamma<T, NX, NY> g;
     g.load_transition(gview<T>(a), s);
     T mf[NX];
     load<T, NX>((const T*)a.mf + e * NX, mf);
-    T df[X], gb[GR::size];
+    T gb[GR::size];
     // FP32 holds the record in registers; FP64 reads it where it is used
     // (twice the registers per value would spill).
     T rtr[sizeof(T) == 4 ? RT::size : 4];
     if constexpr (sizeof(T) == 4) vload<T, RT::size>(rtg, rtr);
     const T* rt = sizeof(T) == 4 ? rtr : rtg;
     rts_vjp<T, NX, NY>(rt, g.F, mf, x, df, gb);
-    store<T, X>((T*)a.dfilt + e * X, df);
     store<T, NX * NX>(go + GR::F, gb + GR::F);
     store<T, NX>(go + GR::c, gb + GR::c);
     store<T, NX * NX>(go + GR::L, gb + GR::L);
@@ -181,14 +205,18 @@ adj_smoother_leaf_down(DevLevel lv, int leaf, bool per_step, DevSeqs sq, AdjBufs
     smoother_adj_map<T, NX>(G, (const T*)a.dir + (e + 1) * X, mp);
     map_apply<T, NX>(mp, x, xn);
     copy<T, X>(xn, x);
-    if (s == last) store<T, X>((T*)a.dfilt + (e + 1) * X, x);   // k = n: dmf_n = x_n
   };
+  T* dfilt = (T*)a.dfilt;
   T* gbar = (T*)a.gbar;
   if (!per_step) {   // one thread walks its whole chunk
     if (!active) return;
     for (int j = 0; j < cnt; ++j) {
-      vjp(j, gbar + (s0 + j) * GR::size);
-      if (j + 1 < cnt || s0 + j == last) advance(j);
+      const int64_t s = s0 + j;
+      T df[X];
+      vjp(j, (const T*)a.rtab + s * RT::size, gbar + s * GR::size, df);
+      store<T, X>(dfilt + (s + b) * X, df);
+      if (j + 1 < cnt || s == last) advance(j);
+      if (s == last) store<T, X>(dfilt + (s + b + 1) * X, x);   // k = n: dmf_n = x_n
     }
     return;
   }
@@ -196,36 +224,70 @@ adj_smoother_leaf_down(DevLevel lv, int leaf, bool per_step, DevSeqs sq, AdjBufs
   // step, then all lanes take their VJP together (inside the walk each
   // lane's VJP would come at a different trip and the warp would run it once
   // per distinct step).
-  if (active)
-    for (int j = 0; j < jj; ++j) advance(j);
   const int64_t s = s0 + jj;
   if constexpr (STAGE) {
     // The steps of a warp's active lanes are consecutive and increase with
-    // the lane: their records go out as one block.  The observation part
-    // H | d | Omega is written as zeros here; the filter adjoint, which runs
-    // next, assigns it.
+    // the lane: their records come in and go out as one block.  The
+    // observation part H | d | Omega is written as zeros here; the filter
+    // adjoint, which runs next, assigns it.
     const unsigned mask = __ballot_sync(0xffffffffu, active);
     if (mask == 0) return;   // uniform per warp
-    const int lane = threadIdx.x % kWarp;
-    const int64_t s_lo = __shfl_sync(0xffffffffu, s, __ffs(mask) - 1);
-    const int na = __popc(mask);
-    T* sh = SG + (threadIdx.x / kWarp) * kWarp * GR::size;
+    const int lo = __ffs(mask) - 1, na = __popc(mask), r = __popc(mask & ((1u << lane) - 1));
+    const int64_t s_lo = __shfl_sync(0xffffffffu, s, lo);
+    T* const st = sh + kWarp * RT::size;
+    warp_fetch<4>(sh, (const T*)a.rtab + s_lo * RT::size, na * RT::size);
+    if (active)
+      for (int j = 0; j < jj; ++j) advance(j);
+    warp_fetch_wait();
+    T df[X];
     if (active) {
-      T* rec = sh + (int)(s - s_lo) * GR::size;
-      vjp(jj, rec);
+      T* rec = st + r * GR::size;
+      vjp(jj, sh + r * RT::size, rec, df);
 #pragma unroll
       for (int k = GR::H; k < GR::size; ++k) rec[k] = T(0);
-      if (s == last) advance(jj);
     }
     __syncwarp();
     T* gw = gbar + s_lo * GR::size;
-    for (int k = lane; k < na * GR::size; k += kWarp) gw[k] = sh[k];
+    for (int k = lane; k < na * GR::size; k += kWarp) gw[k] = st[k];
+    // dfilt: a row per step and, after a sequence's last step, its row k = n
+    const bool end = active && s == last;
+    const unsigned ends = __ballot_sync(0xffffffffu, end);
+    const int row = r + __popc(ends & ((1u << lane) - 1)), rows = na + __popc(ends);
+    const int64_t e = s + b, e_lo = __shfl_sync(0xffffffffu, e, lo);
+    // (an empty sequence between two others leaves a row out of the block)
+    const bool block = __all_sync(0xffffffffu, !active || e - e_lo == row);
+    __syncwarp();
+    if (active) {
+      if (end) advance(jj);
+      if (block) {
+        store<T, X>(st + row * X, df);
+        if (end) store<T, X>(st + (row + 1) * X, x);
+      } else {
+        store<T, X>(dfilt + e * X, df);
+        if (end) store<T, X>(dfilt + (e + 1) * X, x);
+      }
+    }
+    if (!block) return;
+    __syncwarp();
+    T* dw = dfilt + e_lo * X;
+    for (int k = lane; k < rows * X; k += kWarp) dw[k] = st[k];
   } else {
     if (active) {
-      vjp(jj, gbar + s * GR::size);
-      if (s == last) advance(jj);
+      T df[X];
+      for (int j = 0; j < jj; ++j) advance(j);
+      vjp(jj, (const T*)a.rtab + s * RT::size, gbar + s * GR::size, df);
+      store<T, X>(dfilt + (s + b) * X, df);
+      if (s == last) {
+        advance(jj);
+        store<T, X>(dfilt + (s + b + 1) * X, x);
+      }
     }
   }
+}
+
+// Dynamic shared memory of adj_smoother_leaf_down's blocks.
+template <typename T> constexpr size_t adj_leaf_down_smem(bool per_step) {
+  return sizeof(T) == 4 && per_step ? kBlock * sizeof(T) * (RtsTab<5>::size + GRec<5, 2>::size) : 0;
 }
 
 // --------------------------- filter adjoint (backward in time) ------------
@@ -330,13 +392,12 @@ adj_filter_leaf_down(DevLevel lv, int leaf, bool per_step, DevSeqs sq, AdjBufs a
   }
   // One thread per step: the lanes walk their maps first and take their VJPs
   // together (as in adj_smoother_leaf_down).
-  if (active)
-    for (int j = cnt - 1; j > jj; --j) advance(j);
   const int64_t s = s0 + jj;
   if constexpr (STAGE) {
     // The steps of a warp's active lanes are consecutive and increase with
     // the lane (chunks of consecutive steps; only a sequence's last chunk is
-    // short): their records are read and written as one block.
+    // short): their records are read and written as one block, fetched while
+    // the lanes walk their maps (512000 steps 183 -> 157 us).
     const unsigned mask = __ballot_sync(0xffffffffu, active);
     if (mask == 0) return;   // uniform per warp
     const int lane = threadIdx.x % kWarp;
@@ -344,13 +405,18 @@ adj_filter_leaf_down(DevLevel lv, int leaf, bool per_step, DevSeqs sq, AdjBufs a
     const int na = __popc(mask);
     T* sh = SG + (threadIdx.x / kWarp) * kWarp * GR::size;
     T* gw = gbar + s_lo * GR::size;
-    for (int k = lane; k < na * GR::size; k += kWarp) sh[k] = gw[k];
-    __syncwarp();
+    warp_fetch<1>(sh, gw, na * GR::size);
+    if (active)
+      for (int j = cnt - 1; j > jj; --j) advance(j);
+    warp_fetch_wait();
     if (active) vjp(jj, sh + (int)(s - s_lo) * GR::size);
     __syncwarp();
     for (int k = lane; k < na * GR::size; k += kWarp) gw[k] = sh[k];
   } else {
-    if (active) vjp(jj, gbar + s * GR::size);
+    if (active) {
+      for (int j = cnt - 1; j > jj; --j) advance(j);
+      vjp(jj, gbar + s * GR::size);
+    }
   }
 }
 
