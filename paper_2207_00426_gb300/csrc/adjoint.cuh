@@ -545,8 +545,9 @@ SQSM_DEV void kf_vjp(const KfQ<T, NX, NY>& q, const Gamma<T, NX, NY>& g, const T
 // the form of the forward kernel): given cotangents Gb of the regression
 // matrix, ob of the offset (absolute form z_bar - G m) and Lb of the noise
 // covariance, accumulate into mb, Nb.  JAC(x, J) writes the Jacobian of
-// the regressed function at x; G, s (residual columns) are recomputed.
-template <typename T, int NO, typename JAC>
+// the regressed function at x; it depends on the first MOVE components, which
+// only the first MOVE columns of the lower factor N change.
+template <typename T, int NO, int MOVE, typename JAC>
 SQSM_DEV void cubature_vjp(const T* m, const T* N, const T* G, const T* sres, const T* Gb,
                            const T* ob, const T* Lb, JAC jac, T* mb, T* Nb) {
   constexpr int NX = 5;
@@ -590,26 +591,39 @@ SQSM_DEV void cubature_vjp(const T* m, const T* N, const T* G, const T* sres, co
   T common[NO];
 #pragma unroll
   for (int r = 0; r < NO; ++r) common[r] = (ob[r] - sum[r]) / T(2 * NX);
+  T J0[NO * NX];
+  if constexpr (MOVE < NX) jac(m, J0);
 #pragma unroll
   for (int i = 0; i < NX; ++i) {
-    T X[NX], J[NO * NX], zp[NO], zn[NO], xp[NX], xn[NX];
+    // the pair m +- sq N e_i, one code for both: ten copies of the Jacobian
+    // (a sincos and its branches in each) waited on instruction fetch
+    T add[NX], sub[NX];
+#pragma unroll 1
+    for (int neg = 0; neg < 2; ++neg) {
+      const T sg = neg ? T(-1) : T(1), ssq = sg * sq;
+      T X[NX], J[NO * NX], z[NO], x[NX];
 #pragma unroll
-    for (int r = 0; r < NO; ++r) {
-      zp[r] = Db[r * NX + i] / (T(2) * sq) + T(0.5) * sb[r * NX + i] + common[r];
-      zn[r] = -Db[r * NX + i] / (T(2) * sq) + T(0.5) * sb[r * NX + i] + common[r];
+      for (int r = 0; r < NO; ++r)
+        z[r] = sg * (Db[r * NX + i] / (T(2) * sq)) + T(0.5) * sb[r * NX + i] + common[r];
+      if (i < MOVE) {
+#pragma unroll
+        for (int j = 0; j < NX; ++j) X[j] = m[j] + ssq * N[j * NX + i];
+        jac(X, J);
+      } else {
+#pragma unroll
+        for (int k = 0; k < NO * NX; ++k) J[k] = J0[k];
+      }
+      mtv<T, NO, NX>(J, z, x);
+#pragma unroll
+      for (int j = 0; j < NX; ++j) {
+        add[j] = neg ? add[j] + x[j] : x[j];
+        sub[j] = neg ? sub[j] - x[j] : x[j];
+      }
     }
 #pragma unroll
-    for (int j = 0; j < NX; ++j) X[j] = m[j] + sq * N[j * NX + i];
-    jac(X, J);
-    mtv<T, NO, NX>(J, zp, xp);
-#pragma unroll
-    for (int j = 0; j < NX; ++j) X[j] = m[j] - sq * N[j * NX + i];
-    jac(X, J);
-    mtv<T, NO, NX>(J, zn, xn);
-#pragma unroll
     for (int j = 0; j < NX; ++j) {
-      mb[j] += xp[j] + xn[j];
-      Nb[j * NX + i] += sq * (xp[j] - xn[j]);
+      mb[j] += add[j];
+      Nb[j * NX + i] += sq * sub[j];
     }
   }
 }

@@ -618,7 +618,7 @@ SQSM_DEV void adj_slr_row(int64_t e, int b, const DevSeqs& sq, const CTParams<T>
     if constexpr (LIN == 0) {
       T t[ST::obs];
       vload<T, ST::obs>((const T*)a.stab + s * ST::size, t);
-      cubature_vjp<T, NX>(m, N, t + ST::Gf, t + ST::sf, gb + GR::F, gb + GR::c, Lb, jf, mb, Nb);
+      cubature_vjp<T, NX, NX>(m, N, t + ST::Gf, t + ST::sf, gb + GR::F, gb + GR::c, Lb, jf, mb, Nb);
     } else if constexpr (LIN == 1) {
       taylor_vjp<T, NX>(m, gb + GR::F, gb + GR::c,
                         [&](const T* xx, const T* Jb, T* o) { ct_jac_f_vjp(P, xx, Jb, o); }, mb);
@@ -649,7 +649,7 @@ SQSM_DEV void adj_slr_row(int64_t e, int b, const DevSeqs& sq, const CTParams<T>
     if constexpr (LIN == 0) {
       T t[ST::size - ST::obs];
       vload<T, ST::size - ST::obs>((const T*)a.stab + s * ST::size + ST::obs, t);
-      cubature_vjp<T, NY>(m, N, t + (ST::Gh - ST::obs), t + (ST::sh - ST::obs), gb + GR::H,
+      cubature_vjp<T, NY, 2>(m, N, t + (ST::Gh - ST::obs), t + (ST::sh - ST::obs), gb + GR::H,
                           gb + GR::d, Lb, jh, mb, Nb);
     } else if constexpr (LIN == 1) {
       taylor_vjp<T, NY>(m, gb + GR::H, gb + GR::d,
