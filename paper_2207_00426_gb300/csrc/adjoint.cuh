@@ -597,6 +597,8 @@ SQSM_DEV void cubature_vjp(const T* m, const T* N, const T* G, const T* sres, co
   for (int i = 0; i < NX; ++i) {
     // the pair m +- sq N e_i, one code for both: ten copies of the Jacobian
     // (a sincos and its branches in each) waited on instruction fetch
+    // (512000 steps in FP32 192 -> 180 us, FP64 gradient of 64 x 1000 steps
+    // 28.1 -> 20.2 ms with the FP64 scan's other changes)
     T add[NX], sub[NX];
 #pragma unroll 1
     for (int neg = 0; neg < 2; ++neg) {
