@@ -174,7 +174,9 @@ SQSM_DEV void tria(T* a) {
     const T s2 = s2a + s2b;
     T x0 = T(0);
     if constexpr (pivot >> i & 1) x0 = a[i * C + i];
-    const bool nz = s2 > Tiny<T>::value;
+    // (a NaN is no zero row: L_ii carries it on, also where no other entry of
+    // the factor would read that column)
+    const bool nz = !(s2 <= Tiny<T>::value);
     const T alpha = hh_sqrt(nz ? s2 : T(1));
     const T sgn = x0 >= T(0) ? T(1) : T(-1);
     const T v0 = x0 + sgn * alpha;
