@@ -48,11 +48,14 @@ SQSM_DEV double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 SQSM_DEV float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 SQSM_DEV double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// x / c for a constant c: the product with the rounded reciprocal, corrected
-// by the remainder (a division by a divisor known in advance; Brisebarre,
-// Muller and Raina, IEEE Trans. Computers 2004).  Equal to the rounded
-// quotient: for the divisors the sigma-point rules use (10, 12 and once and
-// twice sqrt(5), sqrt(6)) checked over every FP32 significand.
+// x / c for a constant c > 1: the product with the rounded reciprocal,
+// corrected by the remainder (a division by a divisor known in advance;
+// Brisebarre, Muller and Raina, IEEE Trans. Computers 2004).  Equal to the
+// rounded quotient, for the divisors the sigma-point rules use (10, 12 and
+// once and twice sqrt(5), sqrt(6)) and away from underflow: in FP32 checked
+// over every significand, in FP64 over every one whose quotient is near enough
+// to a rounding boundary for the correction's error to matter.  An infinite x
+// has no remainder and gives the product.
 template <typename T> struct ConstDivisor {
   T c, rc;
   __host__ __device__ constexpr explicit ConstDivisor(T c_) : c(c_), rc(T(1) / c_) {}
@@ -60,7 +63,8 @@ template <typename T> struct ConstDivisor {
 template <typename T>
 SQSM_DEV T div_const(T x, const ConstDivisor<T>& d) {
   const T q = mul_rn(x, d.rc);
-  return fma_rn(fma_rn(-q, d.c, x), d.rc, q);
+  const T r = fma_rn(fma_rn(-q, d.c, x), d.rc, q);
+  return isfinite(q) ? r : q;
 }
 
 // Which entries of a matrix handed to Tria can be nonzero: row(i) is the bit

@@ -1,6 +1,7 @@
 """A NaN in an input reaches the results of the steps that depend on it: the
 factorisation's structural zeros leave out products with exact zeros, never a
-row's own entry."""
+row's own entry.  A difference of sigma points that overflows divides to
+infinity."""
 import numpy as np
 import pytest
 
@@ -38,3 +39,21 @@ def test_nan_in_last_noise_entry(B, dt, nx, ny, n, leaf, key):
     assert bool(torch.isnan(ll).all())
     assert ctx.status() & B.ERR_NONFINITE
     ctx.close()
+
+
+@pytest.mark.parametrize("rule", ["CUBATURE", "UNSCENTED"])
+def test_overflowing_difference_stays_infinite(B, rule):
+    """FP64, a turn of 1 rad per step and a spread of 7e307 of v_x: the points'
+    v_y are +- s sin(1) 7e307 (s^2 = 5 or 6), both finite; their difference
+    overflows, and the regression's F[v_y][v_x] = inf / (2 s) / 7e307 is
+    infinite."""
+    f64, big = torch.float64, 7e307
+    ms = torch.zeros((2, 5), dtype=f64, device="cuda:0")
+    ms[:, 4] = 100.0                    # dt = 0.01
+    Ns = 1e-3 * torch.eye(5, dtype=f64, device="cuda:0").repeat(2, 1, 1)
+    Ns[0, 2, 2] = big
+    F = B.sqsm_ct_linearize(B.Context(0), W.CT_THETA_TRUE,
+                            torch.zeros((1, 2), dtype=f64, device="cuda:0"), [0, 1], ms, Ns,
+                            getattr(B, rule))[0]
+    torch.cuda.synchronize()
+    assert F[0, 3, 2].item() == float("inf")
