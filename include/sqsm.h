@@ -126,8 +126,9 @@ typedef struct {
  * autotune = 1 (with leaf_chunk = radix = 0): the first sqsm_ipls_smooth or
  * sqsm_ipls_nll_grad call of each workload shape (dtype, linearisation,
  * batch size, log2 of the total and of the longest sequence length) times
- * one IPLS iteration for each candidate scan shape on the caller's inputs
- * and stream, keeps the fastest for the context, then runs the call.  That
+ * one IPLS iteration for each candidate scan shape (from 512 steps on the
+ * default shape among them) on the caller's inputs and stream, keeps the
+ * fastest for the context, then runs the call.  That
  * first call synchronises the stream and overwrites the outputs before
  * writing the final ones; later calls of the shape use the stored choice. */
 typedef struct {
