@@ -43,8 +43,9 @@ void adj_scan_down(const LevelSet& L, const ScanBuffers& W, int top, cudaStream_
 
 template <typename T>
 void adj_enqueue(const IplsArgs& a, const AdjArgs& g, const LevelSet& Lf, const ScanBuffers& Wf,
-                 const LevelSet& Ls, const ScanBuffers& Ws, const ScanBuffers& Wa, DevSeqs sq,
-                 double* partial, int* status, cudaStream_t s) {
+                 const LevelSet& Ls, const ScanBuffers& Ws, const LevelSet& La,
+                 const ScanBuffers& Wa, DevSeqs sq, double* partial, int* status,
+                 cudaStream_t s) {
   constexpr int NX = 5, NY = 2, X = XRec<NX>::size, MREC = MapRec<NX>::size;
   const int64_t rows = Ls.n_items[0];
   // 1. Alg. 3 for M iterations: the nominal trajectory lands in a.ms / a.Ns.
@@ -92,8 +93,8 @@ void adj_enqueue(const IplsArgs& a, const AdjArgs& g, const LevelSet& Lf, const 
   T* lam_b = (T*)g.lam_b;
   cudaMemsetAsync(lam_a, 0, sizeof(T) * X * rows, s);
   cudaMemsetAsync(g.dir, 0, sizeof(T) * X * rows, s);   // step 1 of lam = 0
-  const int Lc = (int)Lf.lv.size();
-  const int Lk = Lf.ks_level(KsMax<T, MREC>::value);
+  const int Lc = (int)La.lv.size();
+  const int Lk = La.ks_level(KsMax<T, MREC>::value);
   const unsigned slr_blocks = grid_for(Ls.lv[0].n_chunks * a.leaf);
   // leaf down-sweeps: one thread per step for short leaf chunks (each replays
   // at most kAdjPerStepMaxLeaf - 1 maps), one per chunk for long ones
@@ -106,22 +107,22 @@ void adj_enqueue(const IplsArgs& a, const AdjArgs& g, const LevelSet& Lf, const 
     if (Lc > 1) {
       adj_smoother_leaf_up<T><<<grid_for(Lf.lv[0].n_chunks), kBlock, 0, s>>>(Lf.lv[0], sq, ab,
                                                                              (T*)Wa.items[1]);
-      adj_scan_up<T, true>(Lf, Wa, Lk, s);
+      adj_scan_up<T, true>(La, Wa, Lk, s);
     } else {
-      cudaMemsetAsync(Wa.flag[Lc], 0, sizeof(int) * Lf.n_items[Lc], s);
+      cudaMemsetAsync(Wa.flag[Lc], 0, sizeof(int) * La.n_items[Lc], s);
     }
-    adj_scan_down<T, true>(Lf, Wa, Lc > 1 ? Lk : Lc, s);
+    adj_scan_down<T, true>(La, Wa, Lc > 1 ? Lk : Lc, s);
     adj_smoother_leaf_down<T><<<down_grid, kBlock, down_smem, s>>>(
         Lf.lv[0], a.leaf, per_step, sq, ab, (const T*)Wa.carry[1], Wa.flag[1]);
     // filter adjoint: backward-in-time scan of maps
     if (Lc > 1) {
       adj_filter_leaf_up<T><<<grid_for(Lf.lv[0].n_chunks), kBlock, 0, s>>>(Lf.lv[0], sq, ab, lbar,
                                                                            (T*)Wa.items[1]);
-      adj_scan_up<T, false>(Lf, Wa, Lk, s);
+      adj_scan_up<T, false>(La, Wa, Lk, s);
     } else {
-      cudaMemsetAsync(Wa.flag[Lc], 0, sizeof(int) * Lf.n_items[Lc], s);
+      cudaMemsetAsync(Wa.flag[Lc], 0, sizeof(int) * La.n_items[Lc], s);
     }
-    adj_scan_down<T, false>(Lf, Wa, Lc > 1 ? Lk : Lc, s);
+    adj_scan_down<T, false>(La, Wa, Lc > 1 ? Lk : Lc, s);
     adj_filter_leaf_down<T><<<down_grid, kBlock, 0, s>>>(
         Lf.lv[0], a.leaf, per_step, sq, ab, lbar, (const T*)Wa.carry[1], Wa.flag[1]);
     // SLR adjoint -> next cotangent of the nominal trajectory (and its direct

@@ -68,6 +68,7 @@ struct Plan {
   std::vector<int64_t> offsets;
   int64_t* d_offsets = nullptr;
   LevelSet filt, smth;
+  LevelSet adj;         // with lanes, levels of the adjoint's scans (ensure_adj)
   std::map<std::pair<int, int>, std::unique_ptr<Workspace>> ws;   // (dtype, nx)
 };
 
@@ -168,18 +169,30 @@ constexpr int64_t kLaneChunkItemsPerSm = 32;
 // Levels of a segmented scan whose level-0 items are `counts[b]` per
 // sequence: chunks of L0 items at the leaf, then chunks of R items (or, for
 // R == 0, of 4 or 32 items chosen per level) until each sequence has one item.
-
+// lane_chunk: items of a lane chunk, 0 for a scan without lane forms.  With
+// `leaf` the leaf chunks are that set's (same counts), tables included.
 bool build_levels(Plan& p, const std::vector<int64_t>& counts0, LevelSet& L, int sm_count,
-                  int lane_chunk) {
+                  int lane_chunk, const LevelSet* leaf = nullptr) {
   std::vector<int64_t> counts = counts0;
+  const bool lanes = p.lanes && lane_chunk > 0;
   L.B = (int)counts0.size();
-  L.lanes = p.lanes;
+  L.lanes = lanes;
   L.leaf = p.L0;
   int level = 0;
   int64_t total = 0;
   for (int64_t v : counts) total += v;
   L.n_items.push_back(total);
   L.cs.assign(1, 0);
+  if (leaf) {
+    L.leaf_chunk_off = leaf->leaf_chunk_off;
+    L.lv.push_back(leaf->lv[0]);
+    L.n_items.push_back(leaf->n_items[1]);
+    L.seq_item_off = {nullptr, leaf->seq_item_off[1]};
+    L.max_seq_items = {0, leaf->max_seq_items[1]};
+    for (auto& v : counts) v = (v + p.L0 - 1) / p.L0;
+    level = 1;
+    if (leaf->lv.size() == 1) return true;   // one leaf chunk per sequence
+  }
   for (;;) {
     int64_t size = level == 0 ? p.L0 : p.R;
     if (level > 0) {
@@ -187,7 +200,7 @@ bool build_levels(Plan& p, const std::vector<int64_t>& counts0, LevelSet& L, int
       if (p.R == 0) {                       // adaptive: see get_plan
         int64_t items = 0;
         for (int64_t v : counts) items += v;
-        if (p.lanes)
+        if (lanes)
           form = items > kLaneMaxItems                   ? kFoldLevel
                  : items > kLaneChunkItemsPerSm * sm_count ? kLaneFoldLevel
                                                            : kLaneChunkLevel;
@@ -431,8 +444,21 @@ bool ensure_refine_tabs(Workspace* w, const Plan* p, int dtype, int nx) {
   return w->ftab != nullptr;
 }
 
-bool ensure_adj(Workspace* w, const Plan* p, int dtype) {
+// The levels of the adjoint's scans: those of the filter, but in a plan with
+// lane forms, whose chunks of 8 items would leave 24 lanes of the adjoint's
+// warps idle and add levels, the ones of a plan without (an adjoint iteration
+// of 8 x 2000 steps 849 -> 713 us, of 16384 977 -> 841).
+const LevelSet& adj_levels(const Plan* p) { return p->lanes ? p->adj : p->filt; }
+
+bool ensure_adj(Workspace* w, Plan* p, int dtype, int sm_count) {
   if (w->adj_ready) return true;
+  if (p->lanes && p->adj.lv.empty()) {
+    std::vector<int64_t> n(p->B);
+    for (int b = 0; b < p->B; ++b) n[b] = p->offsets[b + 1] - p->offsets[b];
+    LevelSet L;
+    if (!build_levels(*p, n, L, sm_count, 0, &p->filt)) return false;
+    p->adj = std::move(L);
+  }
   const size_t es = dtype == SQSM_F64 ? 8 : 4;
   const int64_t rows = p->smth.n_items[0], steps = p->filt.n_items[0];
   const int nx = 5, ny = 2, X = nx + nx * nx;
@@ -459,7 +485,8 @@ bool ensure_adj(Workspace* w, const Plan* p, int dtype) {
   if (!g.nom_m || !g.nom_N || !g.ms2 || !g.Ns2 || !g.dir || !g.dfilt || !g.lam_a || !g.lam_b ||
       !g.gbar || !g.ktab || !g.rtab || !g.stab || !g.th_partial || !g.ll)
     return false;
-  if (!alloc_scan(w->mem, p->filt, w->adj_scan, es * (2 * nx * nx + 2 * nx), es * X)) return false;
+  if (!alloc_scan(w->mem, adj_levels(p), w->adj_scan, es * (2 * nx * nx + 2 * nx), es * X))
+    return false;
   w->adj_ready = true;
   return true;
 }
@@ -1235,7 +1262,7 @@ static int nll_grad_run(sqsm_ctx* ctx, int dtype, const sqsm_model* model, const
   Plan* p = get_plan(ctx, offsets, batch, L0, R, lane_plan(dtype, 5, R));
   if (!p) return fail(ctx, SQSM_ERR_NO_MEMORY, "plan allocation failed");
   Workspace* w = get_ws(p, dtype, 5);
-  if (!w || !ensure_ipls(w, p, dtype) || !ensure_adj(w, p, dtype) ||
+  if (!w || !ensure_ipls(w, p, dtype) || !ensure_adj(w, p, dtype, ctx->sm_count) ||
       (ctx->opt.refine > 0 && !ensure_refine_tabs(w, p, dtype, 5)))
     return fail(ctx, SQSM_ERR_NO_MEMORY, "workspace");
   const void* n0 = prior_input(ctx, w, p, dtype, 5, N0);
@@ -1255,11 +1282,11 @@ static int nll_grad_run(sqsm_ctx* ctx, int dtype, const sqsm_model* model, const
   auto enqueue = [&](cudaStream_t st) {
     enqueue_prior(ctx, p, w, dtype, 5, N0, st);
     if (dtype == SQSM_F32)
-      adj_enqueue_f32(a, adj, p->filt, w->filt, p->smth, w->smth, w->adj_scan, sq, w->partial,
-                      ctx->d_status, st);
+      adj_enqueue_f32(a, adj, p->filt, w->filt, p->smth, w->smth, adj_levels(p), w->adj_scan, sq,
+                      w->partial, ctx->d_status, st);
     else
-      adj_enqueue_f64(a, adj, p->filt, w->filt, p->smth, w->smth, w->adj_scan, sq, w->partial,
-                      ctx->d_status, st);
+      adj_enqueue_f64(a, adj, p->filt, w->filt, p->smth, w->smth, adj_levels(p), w->adj_scan, sq,
+                      w->partial, ctx->d_status, st);
   };
   if (!use_graph) {
     enqueue(s);

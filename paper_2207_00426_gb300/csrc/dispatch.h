@@ -114,12 +114,12 @@ struct AdjArgs {
 };
 void adj_enqueue_f32(const IplsArgs& a, const AdjArgs& g, const LevelSet& Lf,
                      const ScanBuffers& Wf, const LevelSet& Ls, const ScanBuffers& Ws,
-                     const ScanBuffers& Wa, DevSeqs sq, double* partial, int* status,
-                     cudaStream_t s);
+                     const LevelSet& La, const ScanBuffers& Wa, DevSeqs sq, double* partial,
+                     int* status, cudaStream_t s);
 void adj_enqueue_f64(const IplsArgs& a, const AdjArgs& g, const LevelSet& Lf,
                      const ScanBuffers& Wf, const LevelSet& Ls, const ScanBuffers& Ws,
-                     const ScanBuffers& Wa, DevSeqs sq, double* partial, int* status,
-                     cudaStream_t s);
+                     const LevelSet& La, const ScanBuffers& Wa, DevSeqs sq, double* partial,
+                     int* status, cudaStream_t s);
 
 // One SLR pass (Sec. 4.2 / 4.3) of the CT model into caller arrays.
 void ct_linearize_f32(const IplsArgs& a, const LevelSet& Lf, DevSeqs sq, cudaStream_t s);

@@ -16,7 +16,8 @@ namespace sqsm {
 // lanes (lane_scan.cuh): Kogge-Stone chunks of one block, sequential folds of
 // one 16-lane (smoother: 8-lane) group per chunk.  The lane forms hold in a
 // plan made for FP64 and n_x >= kLaneMinNx; another scan over that plan (the
-// adjoint's) takes a lane chunk as a chunk and a lane fold as a fold.
+// refinement's mean-only smoother) takes a lane chunk as a chunk; the
+// gradient's adjoint scans have levels of their own there.
 enum LevelForm { kFoldLevel = 0, kChunkLevel, kLaneChunkLevel, kLaneFoldLevel };
 constexpr int kLaneMinNx = 3;
 

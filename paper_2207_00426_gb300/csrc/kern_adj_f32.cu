@@ -5,9 +5,9 @@ namespace sqsm {
 
 void adj_enqueue_f32(const IplsArgs& a, const AdjArgs& g, const LevelSet& Lf,
                     const ScanBuffers& Wf, const LevelSet& Ls, const ScanBuffers& Ws,
-                    const ScanBuffers& Wa, DevSeqs sq, double* partial, int* status,
-                    cudaStream_t s) {
-  adj_enqueue<float>(a, g, Lf, Wf, Ls, Ws, Wa, sq, partial, status, s);
+                    const LevelSet& La, const ScanBuffers& Wa, DevSeqs sq, double* partial,
+                    int* status, cudaStream_t s) {
+  adj_enqueue<float>(a, g, Lf, Wf, Ls, Ws, La, Wa, sq, partial, status, s);
 }
 
 }  // namespace sqsm
