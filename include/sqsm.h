@@ -189,8 +189,14 @@ typedef struct {
                            changes maxima), and frees each group's
                            workspace before the next group's is made: the
                            call's device memory is then that of one
-                           group, about 3.4 KB per time step in FP32 and
-                           6.6 KB in FP64.  A grouped call runs without
+                           group.  Per time step (1 KB = 1000 bytes) it is
+                           at most 3.5 KB in FP32 (4.1 KB in groups of up to
+                           116736 steps) and in FP64, whose leaf chunks are
+                           shorter in small groups, 10 KB up to 16384
+                           steps, 8.1 KB up to 65536, 7.4 KB up to 116736
+                           and 6.8 KB above (batches of 3-step sequences a
+                           quarter more, any call at least some 10 MB).  A
+                           grouped call runs without
                            graphs and synchronises the device between
                            groups; a sequence longer than the bound
                            returns SQSM_ERR_TOO_LARGE.  0 (default): the
