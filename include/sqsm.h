@@ -206,9 +206,15 @@ typedef struct {
 typedef struct sqsm_ctx sqsm_ctx;
 
 /* The scan shape (leaf_chunk, radix; radix 0 = the adaptive upper levels)
- * that IPLS calls on this context use for a batch of sequences with the
- * given host offsets (batch + 1 values) and dtype: the options', the
- * autotuned choice if one is stored, else the default.  No GPU work. */
+ * that IPLS calls with the given model kind (sqsm_model_kind) use on this
+ * context for a batch of sequences with the given host offsets (batch + 1
+ * values) and dtype: the options', the autotuned choice if one is stored
+ * (coordinated-turn models), else the default, which depends on the model's
+ * n_x.  No GPU work.  SQSM_ERR_INVALID_ARG for an unknown model kind. */
+int sqsm_scan_shape_model(sqsm_ctx* ctx, int model_kind, int dtype, int linearization,
+                          int64_t batch, const int64_t* offsets, int* leaf_chunk, int* radix);
+
+/* sqsm_scan_shape_model of the coordinated-turn models. */
 int sqsm_scan_shape(sqsm_ctx* ctx, int dtype, int linearization, int64_t batch,
                     const int64_t* offsets, int* leaf_chunk, int* radix);
 

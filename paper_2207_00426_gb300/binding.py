@@ -95,6 +95,8 @@ lib.sqsm_kernel_name.restype = ctypes.c_char_p
 lib.sqsm_scan_shape.argtypes = [_p, _int, _int, _i64, ctypes.POINTER(_i64), ctypes.POINTER(_int),
                                 ctypes.POINTER(_int)]
 lib.sqsm_scan_shape.restype = _int
+lib.sqsm_scan_shape_model.argtypes = [_p, _int] + lib.sqsm_scan_shape.argtypes[1:]
+lib.sqsm_scan_shape_model.restype = _int
 lib.sqsm_fp32_fma_probe.argtypes = [_int, _int, _int, _p, ctypes.POINTER(ctypes.c_double), _p]
 lib.sqsm_fp32_fma_probe.restype = _int
 
@@ -102,8 +104,8 @@ EXPORTED = ["sqsm_create", "sqsm_destroy", "sqsm_last_error", "sqsm_get_status",
             "sqsm_supported_shape", "sqsm_lgssm_smooth", "sqsm_ipls_smooth",
             "sqsm_ct_linearize", "sqsm_profile_enable", "sqsm_profile_read",
             "sqsm_kernel_name", "sqsm_lgssm_smooth_noalloc", "sqsm_ipls_nll_grad",
-            "sqsm_scan_shape", "sqsm_ipls_smooth_tol", "sqsm_ipls_smooth_std",
-            "sqsm_fp32_fma_probe"]
+            "sqsm_scan_shape", "sqsm_scan_shape_model", "sqsm_ipls_smooth_tol",
+            "sqsm_ipls_smooth_std", "sqsm_fp32_fma_probe"]
 
 
 class SqsmError(RuntimeError):
@@ -190,13 +192,14 @@ class Context:
         self.check(lib.sqsm_get_status(self.h, ctypes.byref(v)))
         return v.value
 
-    def scan_shape(self, offsets, dtype=torch.float32, linearization=0):
-        """(leaf_chunk, radix) that IPLS calls with these sequence offsets use."""
+    def scan_shape(self, offsets, dtype=torch.float32, linearization=0, model=MODEL_CT_BEARINGS):
+        """(leaf_chunk, radix) that IPLS calls with these sequence offsets and
+        this kind of model use."""
         off = (_i64 * len(offsets))(*[int(v) for v in offsets])
         leaf, radix = _int(0), _int(0)
-        self.check(lib.sqsm_scan_shape(self.h, _dtype_code(dtype), int(linearization),
-                                       len(offsets) - 1, off, ctypes.byref(leaf),
-                                       ctypes.byref(radix)))
+        self.check(lib.sqsm_scan_shape_model(self.h, int(model), _dtype_code(dtype),
+                                             int(linearization), len(offsets) - 1, off,
+                                             ctypes.byref(leaf), ctypes.byref(radix)))
         return leaf.value, radix.value
 
 

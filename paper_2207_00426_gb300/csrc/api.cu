@@ -907,13 +907,18 @@ int choose_ipls_shape(sqsm_ctx* ctx, int dtype, const sqsm_model* model, const d
 
 }  // namespace
 
-extern "C" int sqsm_scan_shape(sqsm_ctx* ctx, int dtype, int linearization, int64_t batch,
-                               const int64_t* offsets, int* leaf_chunk, int* radix) {
+extern "C" int sqsm_scan_shape_model(sqsm_ctx* ctx, int model_kind, int dtype, int linearization,
+                                     int64_t batch, const int64_t* offsets, int* leaf_chunk,
+                                     int* radix) {
   if (!ctx || !leaf_chunk || !radix) return SQSM_ERR_INVALID_ARG;
+  sqsm_model model{};
+  model.kind = model_kind;
+  if (!known_model(&model)) return fail(ctx, SQSM_ERR_INVALID_ARG, "unknown model kind");
   if (batch < 1 || batch > (1 << 30) || !valid_offsets(offsets, batch))
     return fail(ctx, SQSM_ERR_INVALID_ARG, "offsets must start at 0 and increase strictly");
-  default_shape(ctx, dtype, 5, offsets, batch, leaf_chunk, radix);
-  if (ctx->opt.autotune && ctx->opt.leaf_chunk <= 0 && ctx->opt.radix <= 0) {
+  const bool ct = is_ct(&model);
+  default_shape(ctx, dtype, ct ? 5 : 1, offsets, batch, leaf_chunk, radix);
+  if (ct && ctx->opt.autotune && ctx->opt.leaf_chunk <= 0 && ctx->opt.radix <= 0) {
     auto it = ctx->tuned.find(tune_key(dtype, linearization, batch, offsets));
     if (it != ctx->tuned.end()) {
       *leaf_chunk = it->second.first;
@@ -921,6 +926,12 @@ extern "C" int sqsm_scan_shape(sqsm_ctx* ctx, int dtype, int linearization, int6
     }
   }
   return SQSM_OK;
+}
+
+extern "C" int sqsm_scan_shape(sqsm_ctx* ctx, int dtype, int linearization, int64_t batch,
+                               const int64_t* offsets, int* leaf_chunk, int* radix) {
+  return sqsm_scan_shape_model(ctx, SQSM_MODEL_CT_BEARINGS, dtype, linearization, batch, offsets,
+                               leaf_chunk, radix);
 }
 
 int sqsm_ipls_smooth(sqsm_ctx* ctx, int dtype, const sqsm_model* model, const double* theta,
