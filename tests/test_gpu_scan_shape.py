@@ -1,5 +1,5 @@
 """The scan shape that a query reports is the one the calls run with, for every
-kind of model."""
+kind of model, and the default leaf of FP64 coordinated-turn calls."""
 import numpy as np
 import pytest
 
@@ -34,6 +34,23 @@ def test_population_calls_run_the_reported_shape(B, dt, n):
     torch.cuda.synchronize()
     assert all(torch.equal(u, v) for u, v in zip(r[0], r[1]))
     assert not all(torch.equal(u, v) for u, v in zip(r[0], r[2]))
+
+
+@pytest.mark.parametrize("n,leaf", [(1, 1), (16_384, 1), (16_385, 2), (65_536, 2), (65_537, 3)])
+def test_fp64_coordinated_turn_leaf(B, n, leaf):
+    """(these lengths do not depend on the GPU, but 65537 needs 86 SMs)"""
+    f64 = torch.float64
+    ctx = B.Context(0)
+    assert torch.cuda.get_device_properties(0).multi_processor_count >= 86
+    for kind in (B.MODEL_CT_BEARINGS, B.MODEL_CT_BEARINGS_R):
+        assert ctx.scan_shape([0, n], f64, model=kind) == (leaf, 0)
+    y = torch.zeros((n, 2), dtype=f64, device="cuda:0")
+    m0 = torch.zeros((1, 5), dtype=f64, device="cuda:0") + 0.1
+    N0 = 0.1 * torch.eye(5, dtype=f64, device="cuda:0")[None]
+    r = [B.sqsm_ipls_smooth(c, W.CT_THETA_TRUE, y, [0, n], m0, N0, 1, B.EXTENDED)
+         for c in (ctx, B.Context(0, leaf_chunk=leaf))]
+    torch.cuda.synchronize()
+    assert all(torch.equal(u, v) for u, v in zip(*r))
 
 
 def test_unknown_model_is_refused(B):
