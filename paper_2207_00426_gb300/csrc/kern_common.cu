@@ -1,12 +1,13 @@
 // Kernels shared by all paths.
+#include <algorithm>
+
 #include "dispatch.h"
 
 namespace sqsm {
 
-// One block per sequence: strided FP64 partial sums, then a fixed-order
-// shared-memory tree, so the result does not depend on scheduling.
 // Sum of part[lo], part[lo + stride], ... below hi by a block of 256 threads,
-// in a fixed order (valid in thread 0).
+// in a fixed order (strided partial sums, then a tree), so that the result does
+// not depend on scheduling (valid in thread 0).
 __device__ double block_sum(const double* part, int64_t lo, int64_t hi, int64_t stride) {
   __shared__ double buf[256];
   double acc = 0.0;
@@ -20,6 +21,7 @@ __device__ double block_sum(const double* part, int64_t lo, int64_t hi, int64_t 
   return buf[0];
 }
 
+// One block per sequence.
 __global__ void loglik_reduce(DevSeqs sq, const double* __restrict__ partial, int64_t stride,
                               double* __restrict__ loglik, int* status) {
   const int b = blockIdx.x;
@@ -40,17 +42,22 @@ __global__ void loglik_slices(DevSeqs sq, double* partial, int64_t slice) {
   if (threadIdx.x == 0) partial[lo] = v;
 }
 
-// One SM adds a warp of doubles in 19 cycles, so a block per sequence took
-// 13 us for the 33334 chunks of n = 1e5; sequences of more than a slice are
-// summed in slices by many blocks first (7 us, both launches).
+// One SM adds a warp of doubles in 19 cycles, so a block per sequence takes
+// 0.7 us a slice (13 us for the 33334 chunks of n = 1e5), and sequences of
+// more than a slice are summed in slices by many blocks first (7 us, both
+// launches).  The grid has the longest sequence's slices for every sequence
+// (0.6 ns a block, empty or not), and many sequences fill the GPU with a block
+// each: for one sequence of 123 slices among B short ones the sum takes 130 us
+// in one launch at any B up to 3000, and sliced 16 at B = 100, 76 at 1000, 210
+// at 3000, 3998 at 60000 (in one launch 269); for 300 sequences of 4 slices
+// 13 us in one launch, 18 sliced.
 constexpr int64_t kLoglikSlice = 2048;
 
 void enqueue_loglik_reduce(DevSeqs sq, double* partial, int64_t max_chunks, double* loglik,
                            int* status, cudaStream_t s, Prof* P) {
   ProfScope ps(P, K_LOGLIK, s);
   const int64_t slices = (max_chunks + kLoglikSlice - 1) / kLoglikSlice;
-  // (a grid's second dimension holds 65535 blocks)
-  const bool sliced = slices > 1 && sq.B <= 65535;
+  const bool sliced = slices > 1 && sq.B <= std::min<int64_t>(32 * slices, 1000);
   if (sliced) {
     loglik_slices<<<dim3((unsigned)slices, (unsigned)sq.B), 256, 0, s>>>(sq, partial,
                                                                           kLoglikSlice);
