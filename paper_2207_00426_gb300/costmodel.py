@@ -1,24 +1,72 @@
-"""Algorithmic FLOP and byte counts of the kernels, for roofline reporting.
+"""FLOP and byte counts of the kernels, for roofline reporting.
 
-Counts follow the formulas the kernels evaluate (an FMA is 2 flops; an add,
-multiply, divide, square root, log, sine/cosine or atan2 is 1), with the
-triangular structure of the factors taken into account.  Per-launch totals
-use the same chunking as the library's plan (leaf chunks of ``leaf`` steps,
-upper levels of ``radix`` items, or the adaptive 4 / 32 choice for radix 0).
-Upper levels count the work-efficient number of combines (c - 1 per chunk of
-c items); the warp-scanned chunks do more.
+``ipls_kernel_flops`` counts the operations the FP32 kernels execute, once
+each (an FMA is 2 flops; an add, multiply, divide, square root, log,
+sine/cosine or atan2 is 1): the triangular structure of the factors and the
+structural zeros that Tria leaves out are taken into account (``rows``), and
+the sigma points that are not evaluated are not counted.  What threads of one
+combine compute twice counts once; the lane forms of FP64 are not modelled.
+``tria``, ``kf_step`` and ``smoother_element`` without ``rows`` / ``masked``
+count the dense loops.
+
+Per-launch totals use the same chunking as the library's plan (leaf chunks of
+``leaf`` steps, upper levels of ``radix`` items, or the adaptive 4 / 32 choice
+for radix 0).  Upper levels count the work-efficient number of combines (c - 1
+per chunk of c items); the warp-scanned chunks do more.
 """
 import math
 
 
-def tria(R, C, nref=None):
-    """Householder LQ of an R x C block (Tria, Sec. 2.2)."""
+def _ones(mask):
+    return bin(mask).count("1")
+
+
+# Nonzeros of the matrices that Tria takes: row -> bit mask of its columns
+# (the patterns of csrc/linalg.cuh and csrc/ct_model.cuh).
+def dense_then_lower(D):
+    """[X | L], X with D columns."""
+    return lambda i: ((1 << D) - 1) | (((2 << i) - 1) << D)
+
+
+def few_then_identity(K, D):
+    """[X | I], the first K of X's D columns nonzero."""
+    return lambda i: ((1 << K) - 1) | (1 << (D + i))
+
+
+def few_rows_then_identity(K, D):
+    """[X^T | I], the first K of X's D columns nonzero."""
+    return lambda i: ((1 << D) - 1 if i < K else 0) | (1 << (D + i))
+
+
+def few_then_few_lower(K, D):
+    """[X | Y], the first K of X's D columns nonzero, Y's first K full beside a
+    lower triangle."""
+    return lambda i: ((1 << K) - 1) | ((((2 << i) - 1) | ((1 << K) - 1)) << D)
+
+
+def dense_lower_over_lower(K, D):
+    """[[X, S], [N, 0]], K rows of a dense D-column X beside a lower S."""
+    return lambda i: dense_then_lower(D)(i) if i < K else (2 << (i - K)) - 1
+
+
+def bearing_noise(ny, K):
+    """diag(sigma) | K residual columns."""
+    return lambda i: (1 << i) | (((1 << K) - 1) << ny)
+
+
+def tria(R, C, nref=None, rows=None):
+    """Householder LQ of an R x C block (Tria, Sec. 2.2); rows: the columns
+    that can be nonzero (the other entries are not touched)."""
     nref = R if nref is None else nref
+    at = [(1 << C) - 1 if rows is None else rows(i) & ((1 << C) - 1) for i in range(R)]
     f = 0
     for i in range(nref):
-        w = C - i
-        f += 2 * w + 6                      # norm, sqrt, v0, tau
-        f += (R - 1 - i) * (4 * w + 1)      # dot + scale + update per row
+        v = ((at[i] >> i) << i) | (1 << i)
+        f += 2 * _ones(at[i] >> i) + 6      # norm, sqrt, v0, tau
+        for r in range(i + 1, R):           # dot + scale + update per row
+            if at[r] & v:
+                f += 2 * _ones(at[r] & v) + 1 + 2 * _ones(v)
+                at[r] |= v
     return f
 
 
@@ -27,44 +75,73 @@ def tri_mm(M, NX):
     return M * NX * (NX + 1)
 
 
-def kf_step(nx, ny):
+def _mm_lower(nx):
+    """nx x nx times a lower factor; a triangular solve of nx rows costs the same."""
+    return nx * nx * (nx + 1)
+
+
+def _psi(nx, ny):
+    """Tria([[H N^-, S_Omega], [N^-, 0]])."""
+    return tria(nx + ny, nx + ny, rows=dense_lower_over_lower(ny, nx))
+
+
+def kf_step(nx, ny, masked=False):
     W = nx + ny
-    return (2 * nx * nx + nx + tri_mm(nx, nx) + tria(nx, 2 * nx) + tri_mm(ny, nx)
-            + tria(W, W) + ny * (2 * nx + 2) + ny * ny + 4 * ny + 3 + nx * 2 * ny)
+    trias = (tria(nx, 2 * nx, rows=dense_then_lower(nx)) + _psi(nx, ny) if masked
+             else tria(nx, 2 * nx) + tria(W, W))
+    return (2 * nx * nx + nx + tri_mm(nx, nx) + trias + tri_mm(ny, nx)
+            + ny * (2 * nx + 2) + ny * ny + 4 * ny + 3 + nx * 2 * ny)
 
 
 def filter_element(nx, ny):
-    W = nx + ny
-    return (tri_mm(ny, nx) + tria(W, W) + 2 * ny * (2 * nx + 2) + 2 * ny * ny
+    return (tri_mm(ny, nx) + _psi(nx, ny) + 2 * ny * (2 * nx + 2) + 2 * ny * ny
             + 2 * nx * ny + 2 * ny * nx * nx + nx * ny * ny + 2 * nx * nx * ny + 2 * nx * ny)
 
 
-def xi_blocks(nx):
-    """M = U_i^T Z_j (U_i lower), Xi_11 = Tria([M, I]) and the gain
-    G = Z_j M^T Xi_11^{-T} Xi_11^{-1} (product, two triangular solves)."""
-    tri = nx * nx * (nx + 1)            # a triangular solve / product, 2 flops per FMA
-    return tri + tria(nx, 2 * nx) + 2 * nx ** 3 + 2 * tri
+def xi_blocks(nx, nz=None):
+    """M = U_i^T Z_j (U_i lower; Z_j lower, or its first nz columns nonzero),
+    Xi_11 = Tria([M, I]) and the gain G = Z_j M^T Xi_11^{-T} Xi_11^{-1}
+    (product, two triangular solves)."""
+    if nz is None:
+        m = sum(2 * (nx - max(i, j)) for i in range(nx) for j in range(nx))
+        zm = sum(2 * nx * (i + 1) for i in range(nx))
+    else:
+        m, zm = nz * nx * (nx + 1), 2 * nx * nx * nz
+    return (m + tria(nx, 2 * nx, rows=few_then_identity(nz or nx, nx)) + zm
+            + 2 * _mm_lower(nx))
 
 
-def filter_combine(nx):
-    tri = nx * nx * (nx + 1)
-    ab = tri + 4 * nx ** 3 + 2 * (nx * (nx + 1) + nx * nx) + 2 * nx       # I - U G^T, A, b
-    eta = 2 * (3 * nx * nx + nx * (nx + 1)) + 3 * nx
-    u = 2 * nx ** 3 + tri + tria(nx, 2 * nx)                              # A_j U_i Xi_11^{-T}
-    z = tria(nx, 2 * nx) + tri + 2 * nx ** 3 + tria(nx, 2 * nx)            # L, W, A_i^T W
-    return xi_blocks(nx) + ab + eta + u + z
+def filter_combine(nx, nz=None):
+    """Table 3; nz: e_j is a single step's element, Z_j with nz columns (the
+    leaf's folds), else an item of an upper level."""
+    z = nx if nz is None else nz
+    lower = dense_then_lower(nx) if nz is None else few_then_few_lower(z, nx)
+    # I - U_i G^T, A_j (I - U_i G^T), A_ij, b_ij and eta_ij
+    ab = _mm_lower(nx) + 4 * nx ** 3 + filter_combine_means(nx)
+    if nz is not None:      # Z_j Z_j^T b_i: two n_x x nz products, not triangular ones
+        ab += 4 * nx * nz - 2 * nx * (nx + 1)
+    # A_j U_i Xi_11^{-T} and Tria([., U_j]), which FP32 runs in full
+    u = 2 * _mm_lower(nx) + tria(nx, 2 * nx)
+    # L = Tria([M^T, I]), W = Z_j L^{-T}, A_i^T W, Tria([., Z_i])
+    zz = (tria(nx, 2 * nx, rows=few_rows_then_identity(z, nx)) + nx * z * (z + 1)
+          + 2 * nx * nx * z + tria(nx, 2 * nx, rows=lower))
+    return xi_blocks(nx, nz) + ab + u + zz
 
 
 def filter_apply(nx):
-    tri = nx * nx * (nx + 1)
-    b = 2 * (nx * (nx + 1) + 2 * nx * nx) + 3 * nx
-    return xi_blocks(nx) + b + 2 * nx ** 3 + tri + tria(nx, 2 * nx)
+    """Table 3 with A_i = 0: b_ij and U_ij alone."""
+    b = 3 * nx * (nx + 1) + 4 * nx * nx + 3 * nx
+    return xi_blocks(nx) + b + 2 * _mm_lower(nx) + tria(nx, 2 * nx)
 
 
-def smoother_element(nx):
-    return (tri_mm(nx, nx) + tria(2 * nx, 2 * nx) + nx ** 3 + 4 * nx * nx + 2 * nx)
+def smoother_element(nx, masked=False):
+    # (n_x <= 2: the loops in full)
+    phi = tria(2 * nx, 2 * nx,
+               rows=dense_lower_over_lower(nx, nx) if masked and nx > 2 else None)
+    return tri_mm(nx, nx) + phi + nx ** 3 + 4 * nx * nx + 2 * nx
 
 
+# (FP32 runs these two Trias in full)
 def smoother_combine(nx):
     return 2 * nx ** 3 + 2 * nx * nx + nx + tri_mm(nx, nx) + tria(nx, 2 * nx)
 
@@ -105,16 +182,19 @@ def filter_combine_means(nx):
 
 # CT cubature SLR: per sigma point the transition difference costs two turn
 # coefficient evaluations (sincos x2, series or divide) and ~24 flops; a
-# bearing difference costs ~8 flops + atan2 per sensor.
+# bearing difference costs ~8 flops + atan2 per sensor, and only the points of
+# the first two columns move the bearings.
 CT_F_DELTA = 2 * 12 + 24
 CT_H_DELTA = 2 * (9 + 1)
+CT_H_COLS = 2
 
 
 def slr_cubature_ct(nx=5, ny=2):
+    nc = CT_H_COLS
     tr = (20 + 2 * nx * CT_F_DELTA + nx * nx * 4 + nx * nx * nx + 2 * nx * nx
           + nx * (2 * nx) + tria(nx, 2 * nx))
-    ob = (2 * 10 + 2 * nx * CT_H_DELTA + ny * nx * 4 + ny * nx * nx + 2 * ny * nx
-          + ny * (nx + ny) + tria(ny, ny + nx) + 2 * 4)
+    ob = (2 * 10 + 2 * nc * CT_H_DELTA + ny * nc * 4 + ny * nc * nc + 2 * ny * nc
+          + ny * (nx + ny) + tria(ny, ny + nx, rows=bearing_noise(ny, nx)) + 2 * 4)
     return tr + ob
 
 
@@ -176,14 +256,15 @@ def ipls_kernel_flops(lengths, nx=5, ny=2, leaf=None, radix=0, linearization="cu
     fl = _levels(lengths, leaf, radix)
     sl = _levels([n + 1 for n in lengths], leaf, radix)
     fe, fc, fa = filter_element(nx, ny), filter_combine(nx), filter_apply(nx)
+    fs = filter_combine(nx, min(nx, ny))
     if len(fl) > 1:
-        out["filter_leaf_up"] = (sum(c * fe + (c - 1) * fc for c in fl[0]), 1)
+        out["filter_leaf_up"] = (sum(c * fe + (c - 1) * fs for c in fl[0]), 1)
     ups = [sum((c - 1) * fc for c in lv) for lv in fl[1:]]
     downs = [sum((c - 1) * fa for c in lv) for lv in fl[1:]]
     if ups:
         out["filter_up"] = (sum(ups) / len(ups), len(ups))
         out["filter_down"] = (sum(downs) / len(downs), len(downs))
-    out["filter_leaf_down"] = (nsteps * kf_step(nx, ny), 1)
+    out["filter_leaf_down"] = (nsteps * kf_step(nx, ny, masked=True), 1)
     nel = nsteps + len(lengths)
 
     def smoother(se, sc, sa):
@@ -198,7 +279,7 @@ def ipls_kernel_flops(lengths, nx=5, ny=2, leaf=None, radix=0, linearization="cu
             sm["smoother_down"] = (sum(downs) / len(downs), len(downs))
         sm["smoother_leaf_down"] = ((nel - len(lengths)) * (se + sa), 1)
         return sm
-    full = smoother(smoother_element(nx), smoother_combine(nx), smoother_apply(nx))
+    full = smoother(smoother_element(nx, masked=True), smoother_combine(nx), smoother_apply(nx))
     out.update(full)
     if refine:
         # each refinement pass: the filter scan again (its small upper levels
