@@ -21,6 +21,8 @@ namespace sqsm {
 enum LevelForm { kFoldLevel = 0, kChunkLevel, kLaneChunkLevel, kLaneFoldLevel };
 constexpr int kLaneMinNx = 3;
 
+// (their scans then have no kChunkLevel: a plan for them with adaptive levels
+// has lane forms, one with an explicit radix folds)
 template <typename T, int NX> constexpr bool lane_forms() {
   return sizeof(T) == 8 && NX >= kLaneMinNx && NX <= kLaneRows;
 }
@@ -283,10 +285,14 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
           continue;
         }
       }
-      if (L.chunk_scan(l))
-        filter_up_cs<T, NX><<<(unsigned)L.lv[l].n_chunks, kChunkScan, 0, s>>>(
-            L.lv[l], (T*)W.items[l], (T*)W.items[l + 1]);
-      else if (L.lv[l].n_chunks <= kWarpLevelMaxChunks)
+      if constexpr (!lane_forms<T, NX>()) {
+        if (L.chunk_scan(l)) {
+          filter_up_cs<T, NX><<<(unsigned)L.lv[l].n_chunks, kChunkScan, 0, s>>>(
+              L.lv[l], (T*)W.items[l], (T*)W.items[l + 1]);
+          continue;
+        }
+      }
+      if (L.lv[l].n_chunks <= kWarpLevelMaxChunks)
         filter_up_w<T, NX><<<wgrid_for(L.lv[l].n_chunks), kWarp * kWarpsPerBlock, 0, s>>>(
             L.lv[l], (const T*)W.items[l], (T*)W.items[l + 1]);
       else
@@ -321,7 +327,7 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
   } else {
     cudaMemsetAsync(W.flag[Lc], 0, sizeof(int) * L.n_items[Lc], s);
   }
-  const bool fused = Lc > 1 && fuse_down(L, Lk);
+  const bool fused = !lane_forms<T, NX>() && Lc > 1 && fuse_down(L, Lk);
   for (int l = (Lc > 1 ? Lk : Lc) - 1; l >= (fused ? 2 : 1); --l) {
     ProfScope ps(P, K_FILTER_DOWN, s);
     if constexpr (lane_forms<T, NX>()) {
@@ -337,12 +343,15 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
             (T*)W.carry[l], W.flag[l]);
         continue;
       }
+    } else {
+      if (L.chunk_scan(l)) {
+        filter_down_cs<T, NX><<<cs_down_grid(L.lv[l].n_chunks), kBlock, 0, s>>>(
+            L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1], W.flag[l + 1],
+            (T*)W.carry[l], W.flag[l]);
+        continue;
+      }
     }
-    if (L.chunk_scan(l))
-      filter_down_cs<T, NX><<<cs_down_grid(L.lv[l].n_chunks), kBlock, 0, s>>>(
-          L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1], W.flag[l + 1],
-          (T*)W.carry[l], W.flag[l]);
-    else if (L.lv[l].n_chunks <= kWarpLevelMaxChunks)
+    if (L.lv[l].n_chunks <= kWarpLevelMaxChunks)
       filter_down_w<T, NX><<<wgrid_for(L.lv[l].n_chunks), kWarp * kWarpsPerBlock, 0, s>>>(
           L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1], W.flag[l + 1],
           (T*)W.carry[l], W.flag[l]);
@@ -352,12 +361,15 @@ void enqueue_filter(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv,
           (T*)W.carry[l], W.flag[l]);
   }
   ProfScope ps(P, K_FILTER_LEAF_DOWN, s);
-  if (fused)
-    filter_down_leaf<T, NX, NY, GV, FO><<<cs_down_grid(L.lv[1].n_chunks), kBlock, 0, s>>>(
-        L.lv[1], (const T*)W.items[1], (const T*)W.carry[2], W.flag[2], L.lv[0], sq, gv, y, m0, N0,
-        fo, partial, status);
-  else
-    filter_leaf_down<T, NX, NY, GV, FO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
+  if constexpr (!lane_forms<T, NX>()) {
+    if (fused) {
+      filter_down_leaf<T, NX, NY, GV, FO><<<cs_down_grid(L.lv[1].n_chunks), kBlock, 0, s>>>(
+          L.lv[1], (const T*)W.items[1], (const T*)W.carry[2], W.flag[2], L.lv[0], sq, gv, y, m0,
+          N0, fo, partial, status);
+      return;
+    }
+  }
+  filter_leaf_down<T, NX, NY, GV, FO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
       L.lv[0], sq, gv, y, m0, N0, (const T*)W.carry[1], W.flag[1], fo, partial, status);
 }
 
@@ -397,11 +409,14 @@ void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv
               L.lv[l], (const T*)W.items[l], (T*)W.items[l + 1]);
           continue;
         }
+      } else {
+        if (L.chunk_scan(l)) {
+          smoother_up_cs<T, NX><<<(unsigned)L.lv[l].n_chunks, kChunkScan, 0, s>>>(
+              L.lv[l], (T*)W.items[l], (T*)W.items[l + 1]);
+          continue;
+        }
       }
-      if (L.chunk_scan(l))
-        smoother_up_cs<T, NX><<<(unsigned)L.lv[l].n_chunks, kChunkScan, 0, s>>>(
-            L.lv[l], (T*)W.items[l], (T*)W.items[l + 1]);
-      else if (L.lv[l].n_chunks <= kWarpLevelMaxChunks)
+      if (L.lv[l].n_chunks <= kWarpLevelMaxChunks)
         smoother_up_w<T, NX><<<wgrid_for(L.lv[l].n_chunks), kWarp * kWarpsPerBlock, 0, s>>>(
             L.lv[l], (const T*)W.items[l], (T*)W.items[l + 1]);
       else
@@ -423,7 +438,7 @@ void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv
   } else {
     cudaMemsetAsync(W.flag[Lc], 0, sizeof(int) * L.n_items[Lc], s);
   }
-  const bool fused = Lc > 1 && fuse_down(L, Lk);
+  const bool fused = !lane_forms<T, NX>() && Lc > 1 && fuse_down(L, Lk);
   for (int l = (Lc > 1 ? Lk : Lc) - 1; l >= (fused ? 2 : 1); --l) {
     ProfScope ps(P, K_SMOOTHER_DOWN, s);
     if constexpr (lane_forms<T, NX>()) {
@@ -440,12 +455,15 @@ void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv
             (T*)W.carry[l], W.flag[l]);
         continue;
       }
+    } else {
+      if (L.chunk_scan(l)) {
+        smoother_down_cs<T, NX><<<cs_down_grid(L.lv[l].n_chunks), kBlock, 0, s>>>(
+            L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1], W.flag[l + 1],
+            (T*)W.carry[l], W.flag[l]);
+        continue;
+      }
     }
-    if (L.chunk_scan(l))
-      smoother_down_cs<T, NX><<<cs_down_grid(L.lv[l].n_chunks), kBlock, 0, s>>>(
-          L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1], W.flag[l + 1],
-          (T*)W.carry[l], W.flag[l]);
-    else if (L.lv[l].n_chunks <= kWarpLevelMaxChunks)
+    if (L.lv[l].n_chunks <= kWarpLevelMaxChunks)
       smoother_down_w<T, NX><<<wgrid_for(L.lv[l].n_chunks), kWarp * kWarpsPerBlock, 0, s>>>(
           L.lv[l], (const T*)W.items[l], (const T*)W.carry[l + 1], W.flag[l + 1],
           (T*)W.carry[l], W.flag[l]);
@@ -470,13 +488,16 @@ void enqueue_smoother(const LevelSet& L, const ScanBuffers& W, DevSeqs sq, GV gv
       return;
     }
   }
-  if (fused)
-    smoother_down_leaf<T, NX, NY, GV, FO, SO><<<cs_down_grid(L.lv[1].n_chunks), kBlock, 0, s>>>(
-        L.lv[1], (const T*)W.items[1], (const T*)W.carry[2], W.flag[2], L.lv[0], sq, gv, fo, so,
-        status, add_nominal, dmax, pm);
-  else
-    smoother_leaf_down<T, NX, NY, GV, FO, SO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
-        L.lv[0], sq, gv, fo, (const T*)W.carry[1], W.flag[1], so, status, add_nominal, dmax, pm);
+  if constexpr (!lane_forms<T, NX>()) {
+    if (fused) {
+      smoother_down_leaf<T, NX, NY, GV, FO, SO><<<cs_down_grid(L.lv[1].n_chunks), kBlock, 0, s>>>(
+          L.lv[1], (const T*)W.items[1], (const T*)W.carry[2], W.flag[2], L.lv[0], sq, gv, fo, so,
+          status, add_nominal, dmax, pm);
+      return;
+    }
+  }
+  smoother_leaf_down<T, NX, NY, GV, FO, SO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
+      L.lv[0], sq, gv, fo, (const T*)W.carry[1], W.flag[1], so, status, add_nominal, dmax, pm);
 }
 
 // Record sizes (elements) of the scan buffers.

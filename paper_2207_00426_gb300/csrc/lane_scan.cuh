@@ -36,9 +36,6 @@ constexpr int kLaneFilterChunk = 8;
 constexpr int kLaneSmootherChunk = 16;
 constexpr int kLaneFold = 4;        // items folded by one group at larger levels
 
-SQSM_DEV double lane_rsqrt(double x) { return rsqrt(x); }
-SQSM_DEV float lane_rsqrt(float x) { return rsqrtf(x); }
-
 // Tria([X | Q]) with row r in lane r of each half: x[NX] dense, q[c] the
 // lower Q (c <= r).  l[c] = L[r][c] (0 above the diagonal), rinv[c] =
 // 1 / L[c][c] (0 for a zero row) in every lane; x and q are consumed.
@@ -59,7 +56,7 @@ SQSM_DEV void lane_tria(T* x, T* q, T* l, T* rinv, int r) {
     for (int c = 0; c <= i; ++c) dot += q[c] * qi[c];
     const T s2 = __shfl_sync(kAll, dot, i, kLaneRows);
     const bool nz = s2 > Tiny<T>::value;
-    const T ri = nz ? lane_rsqrt(nz ? s2 : T(1)) : T(0);
+    const T ri = nz ? rsqrt(nz ? s2 : T(1)) : T(0);
     const T li = dot * ri;
     l[i] = r >= i ? li : T(0);
     rinv[i] = ri;

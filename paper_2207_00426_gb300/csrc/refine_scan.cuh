@@ -293,7 +293,7 @@ bool enqueue_smoother_means(const LevelSet& L, const ScanBuffers& W, DevSeqs sq,
     smoother_top_ks_g<T, NX><<<L.B, KS, 0, s>>>(L.seq_item_off[Lk], (const T*)W.items[Lk],
                                                 (T*)W.carry[Lk], W.flag[Lk]);
   }
-  const bool fused = fuse_down(L, Lk);
+  const bool fused = !lane_forms<T, NX>() && fuse_down(L, Lk);
   for (int l = Lk - 1; l >= (fused ? 2 : 1); --l) {
     ProfScope ps(P, K_SMOOTHER_DOWN, s);
     smoother_down_cs_g<T, NX><<<cs_down_grid(L.lv[l].n_chunks), kBlock, 0, s>>>(
@@ -301,12 +301,15 @@ bool enqueue_smoother_means(const LevelSet& L, const ScanBuffers& W, DevSeqs sq,
         (T*)W.carry[l], W.flag[l]);
   }
   ProfScope ps(P, K_SMOOTHER_LEAF_DOWN, s);
-  if (fused)
-    smoother_down_leaf_g<T, NX, NY, GV, FO><<<cs_down_grid(L.lv[1].n_chunks), kBlock, 0, s>>>(
-        L.lv[1], (const T*)W.items[1], (const T*)W.carry[2], W.flag[2], L.lv[0], sq, gv, fo, etab,
-        so, status, pm);
-  else
-    smoother_leaf_down_g<T, NX, NY, GV, FO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
+  if constexpr (!lane_forms<T, NX>()) {
+    if (fused) {
+      smoother_down_leaf_g<T, NX, NY, GV, FO><<<cs_down_grid(L.lv[1].n_chunks), kBlock, 0, s>>>(
+          L.lv[1], (const T*)W.items[1], (const T*)W.carry[2], W.flag[2], L.lv[0], sq, gv, fo,
+          etab, so, status, pm);
+      return true;
+    }
+  }
+  smoother_leaf_down_g<T, NX, NY, GV, FO><<<grid_for(L.lv[0].n_chunks), kBlock, 0, s>>>(
       L.lv[0], sq, gv, fo, etab, (const T*)W.carry[1], W.flag[1], so, status, pm);
   return true;
 }
