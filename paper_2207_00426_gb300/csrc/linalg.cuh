@@ -60,11 +60,14 @@ template <typename T> struct ConstDivisor {
   T c, rc;
   __host__ __device__ constexpr explicit ConstDivisor(T c_) : c(c_), rc(T(1) / c_) {}
 };
+// (in FP64 by the exponent's bits: a comparison would hold the FP64 unit)
+SQSM_DEV bool finite_bits(float x) { return isfinite(x); }
+SQSM_DEV bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 template <typename T>
 SQSM_DEV T div_const(T x, const ConstDivisor<T>& d) {
   const T q = mul_rn(x, d.rc);
   const T r = fma_rn(fma_rn(-q, d.c, x), d.rc, q);
-  return isfinite(q) ? r : q;
+  return finite_bits(q) ? r : q;
 }
 
 // Which entries of a matrix handed to Tria can be nonzero: row(i) is the bit
