@@ -161,7 +161,8 @@ typedef struct {
                            the correction added to the trajectory.  Each
                            pass costs one more filter scan and a smoother
                            scan of the means alone (the factors do not
-                           change; in FP32 with at most 64 sequences and
+                           change; a whole one where levels are folded: in
+                           FP64 from about 5000 steps on; in FP32 with at most 64 sequences and
                            n_x >= 3 the filter scan's top levels too,
                            replayed from what
                            the first pass stores: about 3.4 MB at

@@ -8,12 +8,12 @@
 // the smoothed means change.  These kernels recompute g alone, with the full
 // kernels' operations in the same order (the shared helpers of elements.cuh;
 // E_ij = E_i E_j again by the same product; each element's E_k read from the
-// table the full pass's leaf up-sweep wrote), so the means equal those of a
-// full pass bit for bit while no Tria runs.  The factors already held in the
-// rows are left as the full pass wrote them; the D fields of the scan
-// records and carries are not recomputed (the words these kernels store
-// whole are zeroed or left stale there, and nothing reads them in this
-// pass).
+// table the full pass's leaf up-sweep wrote), so in FP32 the means equal those
+// of a full pass bit for bit while no Tria runs (in FP64 to rounding: the full
+// pass's lane levels bracket otherwise, see engine.cuh).  The factors already
+// held in the rows are left as the full pass wrote them; the D fields of the
+// scan records and carries are not recomputed (the words these kernels store
+// whole are zeroed or left stale there, and nothing reads them in this pass).
 #pragma once
 
 #include "wscan.cuh"
