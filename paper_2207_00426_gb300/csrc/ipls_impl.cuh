@@ -45,17 +45,21 @@ void ipls_phase_model(const IplsArgs& a, const LevelSet& Lf, const ScanBuffers& 
   const int64_t rows = Ls.n_items[0];
   const RowsPacked<T, NX> nom{(T*)a.nrows}, fr{(T*)a.frows};
   if (phase == IPLS_PRE) {
-    ProfScope ps(a.prof, K_INIT, s);
-    if (a.init_ms) {
-      const RowsSplit<T, NX> init{(T*)a.init_ms, (T*)a.init_Ns};
-      rows_convert_kernel<T, NX, true><<<grid_for(rows), kBlock, 0, s>>>(rows, init, nom);
-    } else {
-      broadcast_prior_kernel<T, NX><<<grid_for(Ls.lv[0].n_chunks), kBlock, 0, s>>>(
-          Ls.lv[0], (const T*)a.m0, (const T*)a.N0, nom);
+    {
+      ProfScope ps(a.prof, K_INIT, s);
+      if (a.init_ms) {
+        const RowsSplit<T, NX> init{(T*)a.init_ms, (T*)a.init_Ns};
+        rows_convert_kernel<T, NX, true><<<grid_for(rows), kBlock, 0, s>>>(rows, init, nom);
+      } else {
+        broadcast_prior_kernel<T, NX><<<grid_for(Ls.lv[0].n_chunks), kBlock, 0, s>>>(
+            Ls.lv[0], (const T*)a.m0, (const T*)a.N0, nom);
+      }
     }
-    if (a.centered)
+    if (a.centered) {
+      ProfScope ps(a.prof, K_INIT, s);
       center_prior_kernel<T, NX><<<(sq.B + 127) / 128, 128, 0, s>>>(sq, (const T*)a.m0, nom,
                                                                      (T*)a.dm0);
+    }
     return;
   }
   if (phase == IPLS_POST) {

@@ -55,13 +55,14 @@ constexpr int64_t kLoglikSlice = 2048;
 
 void enqueue_loglik_reduce(DevSeqs sq, double* partial, int64_t max_chunks, double* loglik,
                            int* status, cudaStream_t s, Prof* P) {
-  ProfScope ps(P, K_LOGLIK, s);
   const int64_t slices = (max_chunks + kLoglikSlice - 1) / kLoglikSlice;
   const bool sliced = slices > 1 && sq.B <= std::min<int64_t>(32 * slices, 1000);
   if (sliced) {
+    ProfScope ps(P, K_LOGLIK, s);
     loglik_slices<<<dim3((unsigned)slices, (unsigned)sq.B), 256, 0, s>>>(sq, partial,
                                                                           kLoglikSlice);
   }
+  ProfScope ps(P, K_LOGLIK, s);
   loglik_reduce<<<sq.B, 256, 0, s>>>(sq, partial, sliced ? kLoglikSlice : 1, loglik, status);
 }
 
