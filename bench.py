@@ -399,7 +399,9 @@ def gpu_arm(args, rank, world, local):
             a0[0] += t
             a0[1] += c
     ctx.profile(False)
-    launches_per_step = sum(c for _, c in acc.values()) / nprof + 1   # + parameter kernel
+    # + parameter kernel; the copies of the nominal rows before the refinement
+    # passes are recorded, but are no kernels
+    launches_per_step = sum(c for _, c in acc.values()) / nprof + 1 - M * REFINE
     flops = CM.ipls_kernel_flops([n], leaf=leaf, refine=REFINE)
     total_ms = sum(t for t, _ in acc.values())
     top = max(acc, key=lambda k: acc[k][0])
