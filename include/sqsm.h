@@ -195,7 +195,7 @@ typedef struct {
                            116736 steps) and in FP64, whose leaf chunks are
                            shorter in small groups, 10 KB up to 16384
                            steps, 8.1 KB up to 65536, 7.4 KB up to 116736
-                           and 6.8 KB above (batches of 3-step sequences a
+                           and 6.9 KB above (batches of 3-step sequences a
                            quarter more, any call at least some 10 MB).  A
                            grouped call runs without
                            graphs and synchronises the device between

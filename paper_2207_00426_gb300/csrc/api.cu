@@ -205,7 +205,7 @@ bool build_levels(Plan& p, const std::vector<int64_t>& counts0, LevelSet& L, int
                  : items > kLaneChunkItemsPerSm * sm_count ? kLaneFoldLevel
                                                            : kLaneChunkLevel;
         else
-          form = items <= kFoldAboveItems ? kChunkLevel : kFoldLevel;
+          form = items <= (p.lanes ? kLaneMaxItems : kFoldAboveItems) ? kChunkLevel : kFoldLevel;
         size = form == kChunkLevel ? kChunkScan
                : form == kLaneChunkLevel ? lane_chunk
                : form == kLaneFoldLevel ? kLaneFold : 4;
@@ -446,8 +446,11 @@ bool ensure_refine_tabs(Workspace* w, const Plan* p, int dtype, int nx) {
 
 // The levels of the adjoint's scans: those of the filter, but in a plan with
 // lane forms, whose chunks of 8 items would leave 24 lanes of the adjoint's
-// warps idle and add levels, the ones of a plan without (an adjoint iteration
-// of 8 x 2000 steps 849 -> 713 us, of 16384 977 -> 841).
+// warps idle and add levels, chunks of 32 items below levels of more than
+// kLaneMaxItems, which are folded as the filter's (an adjoint iteration on the
+// filter's levels / with these / with chunks of 32 up to 160000 items: 8 x 2000
+// steps 849 / 713 / 713 us, 40000 1405 / 1258 / 1258, 116736 2137 / 1999 / 2065,
+// 256000 4078 / 3944 / 4391, 300 x 2000 7671 / 7672 / 8608).
 const LevelSet& adj_levels(const Plan* p) { return p->lanes ? p->adj : p->filt; }
 
 bool ensure_adj(Workspace* w, Plan* p, int dtype, int sm_count) {

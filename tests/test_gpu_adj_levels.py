@@ -11,7 +11,8 @@ from paper_2207_00426_gb300 import workloads as W
 
 
 @pytest.mark.parametrize("lengths", [[1], [2, 1, 1], [32], [33], [1024], [1025], [40, 1, 300],
-                                     [1024] * 3 + [1], [1] * 40 + [33], [16384], [16385]])
+                                     [1024] * 3 + [1], [1] * 40 + [33], [16384], [16385],
+                                     [4000] * 10, [4000] * 10 + [2], [999] * 90])
 def test_fp64_gradient_against_folded_levels(lengths):
     from paper_2207_00426_gb300 import binding as B
     f64 = torch.float64
